@@ -204,3 +204,17 @@ def test_traj8_longest_segment_every_key_and_row():
     for name, got, ref in (("dq", dq[b:e, heads], rq), ("dk", dk[b:e, g:g + 1], rk), ("dv", dv[b:e, g:g + 1], rv)):
         err = rel_err(got.float().cpu().numpy(), ref)
         assert err <= REL, (name, err)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 64), (1, 1, 128), (2, 1, 64), (3, 1, 128), (5, 1, 64), (5, 1, 128)])
+def test_query_tile_counts_around_the_rings(hq, hkv, d):
+    """Key tiles with 1 .. 25 query tiles (head by head: 1, 2, 3, 5 of each row block), so that the
+    Q/dO rings, the row-term buffers and the first and last tile of the two chains meet every count,
+    with full and ragged last tiles."""
+    cu = cu_from_lengths([1, 128, 129, 256, 260, 384, 511, 640])
+    q, k, v, do = workloads.draw_dense(77 + d + hq, int(cu[-1]), hq, hkv, d, device="cuda")
+    _, _, dq, dk, dv = run(q, k, v, do, cu)
+    rq, rk, rv = oatt.attn_bwd(q.cpu(), k.cpu(), v.cpu(), do.cpu(), cu)
+    for name, got, ref in (("dq", dq, rq), ("dk", dk, rk), ("dv", dv, rv)):
+        e = rel_err(got.float().cpu().numpy(), ref)
+        assert e <= REL, (name, e)
