@@ -376,8 +376,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                              keep_l2);
         }
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
+    // The whole warp runs the loop and one elected lane issues, so that descriptors and addresses
+    // stay in uniform registers; as a one-lane branch each MMA took 75-100 cycles to issue instead of
+    // the 64 it executes in (four segments of 8,192 at 40/8/128: 1.774 -> 1.674 ms, sixteen of 4,096
+    // at 14/2/64: 0.618 -> 0.562).
       bool ok = mbar_wait(&bars->q_full, 0);
       // descriptors built once; the issue loops only add compile-time offsets
       const uint64_t q0d = smem_desc(sbase + C::OFF_Q0, 16, 1024), q1d = desc_at(q0d, C::TILE);
@@ -403,7 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       uint32_t kaddr = k_off(0), vaddr = 0;  // slot byte offsets of K_{j+1} and V_j
       if (ok) ok = acquire_group(0);
-      if (ok) {
+      if (ok && elect_one()) {
         issue_s<D>(tmem + C::TM_S0, q0d, desc_at(kv_kmaj, kaddr));
         tc_commit(&bars->s_full[0]);
         if (has1) {
@@ -412,6 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if constexpr (GATHER) tc_commit(&bars->kv_empty[0]);
       }
+      __syncwarp();
       // step j reads V_j and K_{j+1}, one group: acquired at the top of the step, one wait a
       // step (a barrier wait stalls the issuing thread for hundreds of cycles while the pipe
       // streams from shared memory, so the fewer the better), a step after the producer asked
@@ -425,30 +430,39 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (j <= m0) {
           if (!mbar_wait(&bars->p_full[0], j & 1)) { ok = false; break; }
           tc_fence_after();
-          issue_pv<D>(tmem + C::TM_O0, tmem + C::TM_S0, desc_at(kv_mnmaj, vaddr), j > 0);
-          if (next && j + 1 <= m0) {
-            issue_s<D>(tmem + C::TM_S0, q0d, desc_at(kv_kmaj, kaddr));
-            tc_commit(&bars->s_full[0]);
-          } else {
-            tc_commit(&bars->o_done[0]);
+          if (elect_one()) {
+            issue_pv<D>(tmem + C::TM_O0, tmem + C::TM_S0, desc_at(kv_mnmaj, vaddr), j > 0);
+            if (next && j + 1 <= m0) {
+              issue_s<D>(tmem + C::TM_S0, q0d, desc_at(kv_kmaj, kaddr));
+              tc_commit(&bars->s_full[0]);
+            } else {
+              tc_commit(&bars->o_done[0]);
+            }
           }
+          __syncwarp();
         }
         // tile 1
         if (has1) {
           if (!mbar_wait(&bars->p_full[1], j & 1)) { ok = false; break; }
           tc_fence_after();
-          issue_pv<D>(tmem + C::TM_O1, tmem + C::TM_S1, desc_at(kv_mnmaj, vaddr), j > 0);
-          if (next) {
-            issue_s<D>(tmem + C::TM_S1, q1d, desc_at(kv_kmaj, kaddr));
-            tc_commit(&bars->s_full[1]);
-          } else {
-            tc_commit(&bars->o_done[1]);
+          if (elect_one()) {
+            issue_pv<D>(tmem + C::TM_O1, tmem + C::TM_S1, desc_at(kv_mnmaj, vaddr), j > 0);
+            if (next) {
+              issue_s<D>(tmem + C::TM_S1, q1d, desc_at(kv_kmaj, kaddr));
+              tc_commit(&bars->s_full[1]);
+            } else {
+              tc_commit(&bars->o_done[1]);
+            }
           }
+          __syncwarp();
         }
         if constexpr (GATHER) {
           // the gathering producer needs its slots back as soon as the MMAs are done with them
-          if (next) tc_commit(&bars->kv_empty[k_item(j + 1) % C::NSLOT]);
-          tc_commit(&bars->kv_empty[v_item(j) % C::NSLOT]);
+          if (elect_one()) {
+            if (next) tc_commit(&bars->kv_empty[k_item(j + 1) % C::NSLOT]);
+            tc_commit(&bars->kv_empty[v_item(j) % C::NSLOT]);
+          }
+          __syncwarp();
         }
       }
       if (!ok) on_timeout(bars, status);
