@@ -260,8 +260,8 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     bwd_main(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
              const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
              const int32_t* __restrict__ cu_seqlens, int32_t num_segments, int32_t num_tokens, int32_t max_seqlen,
-             int32_t hq, int32_t hkv, float scale, float scale_log2, const float* __restrict__ lse,
-             const float* __restrict__ dvec, float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dk,
+             int32_t hq, int32_t hkv, int32_t tail_groups, float scale, float scale_log2,
+             const float* __restrict__ lse, const float* __restrict__ dvec, float* __restrict__ dq_acc, __nv_bfloat16* __restrict__ dk,
              __nv_bfloat16* __restrict__ dv, int32_t* status, const int32_t* __restrict__ tok_gather,
              int32_t traj_tokens, float* __restrict__ dk_acc, float* __restrict__ dv_acc,
              const __grid_constant__ CUtensorMap tm_qr, const __grid_constant__ CUtensorMap tm_kr,
@@ -272,12 +272,20 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
   uint8_t* smem = smem_raw;
   BwdBars* bars = reinterpret_cast<BwdBars*>(smem + C::OFF_BAR);
 
-  // x = key tile (fastest), so the CTAs resident at one time mostly belong to one (segment, kv head)
-  const int sg = (int)(blockIdx.z * 65535u + blockIdx.y);
-  if (sg >= num_segments * hkv) return;
+  // x = key tile (fastest), so the CTAs resident at one time mostly belong to one (segment, kv head).
+  // The last tail_groups of those go key tile by key tile instead, the first (longest) of every
+  // group first: in turn, the last groups' longest CTAs would start when little else is left.
+  int sg = (int)(blockIdx.z * 65535u + blockIdx.y);
+  const int ngroups = num_segments * hkv;
+  if (sg >= ngroups) return;
+  int n = blockIdx.x;  // key tile
+  if (sg >= ngroups - tail_groups) {
+    const int64_t t = (int64_t)(sg - (ngroups - tail_groups)) * gridDim.x + n;
+    n = (int)(t / tail_groups);
+    sg = ngroups - tail_groups + (int)(t % tail_groups);
+  }
   const int seg = sg / hkv;
   const int g = sg - seg * hkv;
-  const int n = blockIdx.x;  // key tile
   const int start = cu_seqlens[seg];
   const int end = cu_seqlens[seg + 1];
   if (start < 0 || end < start || end > num_tokens || end - start > max_seqlen ||
@@ -880,6 +888,15 @@ cudaError_t launch_bwd_d(const AttnArgs& a, const void* o, const float* lse, con
   const int64_t gx = (int64_t)a.num_segments * a.hkv;
   if (gx > (int64_t)65535 * 65535) return cudaErrorInvalidConfiguration;
   dim3 grid((unsigned)ntiles, (unsigned)(gx < 65535 ? gx : 65535), (unsigned)((gx + 65534) / 65535));
+  // Tail: a group of t key tiles is about G t^2 / 2 tiles of work, shared by 152 SMs, and its longest
+  // CTA G t of them; the last `tail_groups` groups are half of what keeps all SMs busy for as long as
+  // the longest CTA of the launch takes (the CTAs before them cover the rest).  8 short rollouts,
+  // 28/4/128: 6.94 ms without, 6.89 / 6.75 / 6.99 / 7.6 with half / this / twice / four times as many
+  // (more groups at once share less in L2); forward + backward at 14/2/64 3.36 -> 3.22.
+  const double tavg = (double)a.num_tokens / ((double)a.num_segments * C::BM);
+  double tail_groups = 152.0 * ntiles / (tavg < 1.0 ? 1.0 : tavg * tavg);
+  if (tail_groups < 1.0) tail_groups = 1.0;
+  if (tail_groups > (double)gx) tail_groups = (double)gx;
   if (ntiles > 0) {
     static std::atomic<int> regs_cache{-1};
     bool regs_ok = false;
@@ -891,8 +908,8 @@ cudaError_t launch_bwd_d(const AttnArgs& a, const void* o, const float* lse, con
     cudaError_t e = cudaFuncSetAttribute(bwd_main<D, GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     bwd_main<D, GATHER><<<grid, C::THREADS, C::SMEM, st>>>(
-        tq, tk, tv, tdo, a.cu_seqlens, a.num_segments, (int32_t)a.num_tokens, a.max_seqlen, a.hq, a.hkv, a.scale,
-        a.scale * 1.4426950408889634f, lse, dvec, GATHER ? dq_t : dq_acc, static_cast<__nv_bfloat16*>(dk),
+        tq, tk, tv, tdo, a.cu_seqlens, a.num_segments, (int32_t)a.num_tokens, a.max_seqlen, a.hq, a.hkv,
+        (int32_t)tail_groups, a.scale, a.scale * 1.4426950408889634f, lse, dvec, GATHER ? dq_t : dq_acc, static_cast<__nv_bfloat16*>(dk),
         static_cast<__nv_bfloat16*>(dv), a.status, a.tok_gather, (int32_t)a.traj_tokens, dk_t, dv_t,
         GATHER ? tqr : tq, GATHER ? tkr : tk, GATHER ? tvr : tv, GATHER ? tqs : tq, GATHER ? tks : tk,
         GATHER ? tvs : tv);
