@@ -138,7 +138,7 @@ vcs_status vcs_plan_segments(const int32_t* cu_steps, int32_t num_traj, int64_t 
   vcs_status s = check_seg_args(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, ws_bytes);
   if (s != VCS_OK) return s;
   SegWorkspace w = seg_workspace_carve(ws, num_traj, num_steps);
-  if (launch_seg_plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, -1, -1, sizes, w,
+  if (launch_seg_plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, w,
                       as_stream(stream)) != cudaSuccess)
     return VCS_ERR_CUDA;
   return VCS_OK;
@@ -157,11 +157,9 @@ vcs_status vcs_build_segments(const int32_t* cu_steps, int32_t num_traj, int64_t
     return VCS_ERR_INVALID_ARG;
   SegWorkspace w = seg_workspace_carve(ws, num_traj, num_steps);
   cudaStream_t st = as_stream(stream);
-  if (launch_seg_plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, seg_capacity, tok_capacity,
-                      sizes, w, st) != cudaSuccess)
-    return VCS_ERR_CUDA;
-  if (launch_seg_build(cu_steps, num_traj, window, keep, step_img, cu_seqlens, seg_traj, tok_gather, tok_src_step,
-                       tok_pos, tok_loss_mask, w, st) != cudaSuccess)
+  if (launch_seg_build(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, seg_capacity, tok_capacity,
+                       cu_seqlens, seg_traj, tok_gather, tok_src_step, tok_pos, tok_loss_mask, sizes, w, st) !=
+      cudaSuccess)
     return VCS_ERR_CUDA;
   return VCS_OK;
 }

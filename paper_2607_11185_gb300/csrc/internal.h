@@ -24,29 +24,30 @@ struct ApiRange {
 
 // ---- segment builder (segments.cu) ----
 struct SegWorkspace {
-  int64_t* step_off;    // [num_steps+1] exclusive prefix of img+txt over all steps
-  int64_t* txt_pre;     // [num_steps+1] exclusive prefix of txt over all steps
-  int32_t* traj_nseg;   // [num_traj]
-  int64_t* traj_ntok;   // [num_traj]
+  int64_t* step_inc;    // [num_steps] per trajectory, inclusive prefix of img+txt over its steps
+  int64_t* txt_inc;     // [num_steps] likewise of txt
   int32_t* traj_maxlen; // [num_traj]
+  int64_t* traj_base;   // [num_traj] first row of each trajectory in the token buffer
   int64_t* seg_base;    // [num_traj+1]
   int64_t* tok_base;    // [num_traj+1]
   int64_t* seg_start;   // [num_steps+1] start of every segment in the packed buffer
   int32_t* seg_full;    // [num_steps] global step of the first full (screenshot) step a_j
   int32_t* seg_new;     // [num_steps] global step of the first new step s_j
   int32_t* seg_last;    // [num_steps] global step of the last step e_j
-  int32_t* seg_first;   // [num_steps] global step of the trajectory's first step
-  int64_t* totals;      // [4]: num_segments, num_tokens, max_seqlen, status
+  int32_t* seg_traj;    // [num_steps] trajectory of the segment
+  int64_t* totals;      // [5]: num_segments, num_tokens, max_seqlen, status, blocks done (256 bytes reserved)
 };
 size_t seg_workspace_bytes(int32_t num_traj, int64_t num_steps);
 SegWorkspace seg_workspace_carve(void* ws, int32_t num_traj, int64_t num_steps);
 
 cudaError_t launch_seg_plan(const int32_t* cu_steps, int32_t num_traj, int64_t num_steps, const int32_t* step_img,
-                            const int32_t* step_txt, int32_t window, int32_t keep, int64_t seg_capacity,
-                            int64_t tok_capacity, vcs_sizes* sizes, const SegWorkspace& w, cudaStream_t st);
-cudaError_t launch_seg_build(const int32_t* cu_steps, int32_t num_traj, int32_t window, int32_t keep,
-                             const int32_t* step_img, int32_t* cu_seqlens, int32_t* seg_traj, int32_t* tok_gather,
-                             int32_t* tok_src_step, int32_t* tok_pos, uint8_t* tok_loss_mask,
+                            const int32_t* step_txt, int32_t window, int32_t keep, vcs_sizes* sizes,
+                            const SegWorkspace& w, cudaStream_t st);
+// plan, segment tables and the per-token expansion
+cudaError_t launch_seg_build(const int32_t* cu_steps, int32_t num_traj, int64_t num_steps, const int32_t* step_img,
+                             const int32_t* step_txt, int32_t window, int32_t keep, int64_t seg_capacity,
+                             int64_t tok_capacity, int32_t* cu_seqlens, int32_t* seg_traj, int32_t* tok_gather,
+                             int32_t* tok_src_step, int32_t* tok_pos, uint8_t* tok_loss_mask, vcs_sizes* sizes,
                              const SegWorkspace& w, cudaStream_t st);
 
 // ---- gather (gather.cu) ----

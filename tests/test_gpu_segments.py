@@ -126,3 +126,25 @@ def test_host_argument_errors():
     assert vcs.vcs_plan_segments(dcu, 1, 2, dimg, dtxt, 0, 0, sizes, ws, nb) == 1      # window 0
     assert vcs.vcs_plan_segments(dcu, 1, 2, dimg, dtxt, 2, -1, sizes, ws, nb) == 1     # keep < 0
     assert vcs.vcs_plan_segments(dcu, 1, 2, dimg, dtxt, 2, 0, sizes, ws, nb - 1) == 8  # workspace
+
+
+@pytest.mark.parametrize("num_traj", [1, 31, 32, 33, 128, 129, 1025, 5000])
+def test_trajectory_counts_around_the_plan_launches(num_traj):
+    # one block plans up to 128 trajectories (32 at a time), more take several blocks and a scan in
+    # chunks of 1,024; up to 70 steps, so that prefix sums and segments exceed a warp's 32 lanes
+    rng = np.random.default_rng(num_traj)
+    t = rng.integers(0, 71 if num_traj < 200 else 6, size=num_traj)
+    cu = np.concatenate([[0], np.cumsum(t)]).astype(np.int32)
+    img = rng.integers(0, 9, size=int(cu[-1])).astype(np.int32)
+    txt = rng.integers(0, 5, size=int(cu[-1])).astype(np.int32)
+    run_and_compare(cu, img, txt, 1, 1)
+
+
+@pytest.mark.parametrize("num_traj", [3, 200])
+def test_inconsistent_data_reported_before_capacity(num_traj):
+    cu = np.arange(num_traj + 1, dtype=np.int32) * 2
+    img = np.full(2 * num_traj, 4, np.int32)
+    txt = np.full(2 * num_traj, 2, np.int32)
+    img[1] = -1
+    st, dst, _, _ = _raw_build(cu, img, txt, 1, 0, 1, 1)
+    assert st == 0 and dst == 6
