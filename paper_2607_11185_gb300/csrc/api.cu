@@ -178,17 +178,9 @@ vcs_status vcs_gather(const void* q_traj, const void* k_traj, const void* v_traj
   for (const void* p : ptrs)
     if (p != nullptr && !aligned16(p)) return VCS_ERR_INVALID_ARG;
   cudaStream_t st = as_stream(stream);
-  if (launch_gather(q_traj, traj_tokens, tok_gather, num_tokens, (int64_t)hq * d * 2, q, dev_status, st) !=
-      cudaSuccess)
+  if (launch_gather(q_traj, k_traj, v_traj, traj_tokens, tok_gather, num_tokens, (int64_t)hq * d * 2,
+                    with_kv ? (int64_t)hkv * d * 2 : 0, q, k, v, dev_status, st) != cudaSuccess)
     return VCS_ERR_CUDA;
-  if (with_kv) {
-    if (launch_gather(k_traj, traj_tokens, tok_gather, num_tokens, (int64_t)hkv * d * 2, k, dev_status, st) !=
-        cudaSuccess)
-      return VCS_ERR_CUDA;
-    if (launch_gather(v_traj, traj_tokens, tok_gather, num_tokens, (int64_t)hkv * d * 2, v, dev_status, st) !=
-        cudaSuccess)
-      return VCS_ERR_CUDA;
-  }
   return VCS_OK;
 }
 

@@ -51,8 +51,10 @@ cudaError_t launch_seg_build(const int32_t* cu_steps, int32_t num_traj, int64_t 
                              const SegWorkspace& w, cudaStream_t st);
 
 // ---- gather (gather.cu) ----
-cudaError_t launch_gather(const void* src, int64_t traj_tokens, const int32_t* tok_gather, int64_t num_tokens,
-                          int64_t row_bytes, void* dst, int32_t* dev_status, cudaStream_t st);
+// kv_row_bytes 0: Q alone
+cudaError_t launch_gather(const void* q_src, const void* k_src, const void* v_src, int64_t traj_tokens,
+                          const int32_t* tok_gather, int64_t num_tokens, int64_t q_row_bytes, int64_t kv_row_bytes,
+                          void* q, void* k, void* v, int32_t* dev_status, cudaStream_t st);
 
 // ---- attention (attn_fwd.cu, attn_bwd.cu) ----
 struct AttnArgs {

@@ -93,3 +93,22 @@ def test_gather_long_horizon_chunk_sampled_rows():
     for src, got in ((q, qs), (k, ks), (v, vs)):
         ref = ogather.gather_rows(src.cpu(), want_map[rows])
         assert torch.equal(got[rows_t].cpu(), ref)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 8), (3, 1, 40), (2, 2, 64), (5, 1, 104), (33, 3, 128), (40, 8, 128)])
+@pytest.mark.parametrize("with_kv", [True, False])
+def test_row_sizes_around_the_warp(hq, hkv, d, with_kv):
+    # rows of 1 .. 640 16-byte chunks: less than a warp's 32, not a multiple of 32 or of 128, whole
+    # 128s; more tokens than warps in the grid
+    from paper_2607_11185_gb300 import vcs
+    g = torch.Generator(device="cuda").manual_seed(hq + d)
+    q, k, v = (torch.randn((777, h, d), generator=g, device="cuda").bfloat16() for h in (hq, hkv, hkv))
+    n = 25001 if hq < 33 else 3001
+    idx = torch.randint(0, 777, (n,), generator=g, device="cuda", dtype=torch.int32)
+    out = [torch.empty((n, h, d), dtype=torch.bfloat16, device="cuda") for h in (hq, hkv, hkv)]
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    kv = (k, v, out[1], out[2]) if with_kv else (None,) * 4
+    assert vcs.vcs_gather(q, kv[0], kv[1], 777, idx, n, hq, hkv, d, out[0], kv[2], kv[3], st) == 0
+    assert int(st.item()) == 0
+    for src, got in zip((q, k, v)[:3 if with_kv else 1], out):
+        assert torch.equal(got, src[idx.long()])
