@@ -186,3 +186,27 @@ def test_group_advantage(group_size):
     a = vcs.group_advantage(r.to(DEV), group_size).cpu().double().numpy()
     want = oloss.group_advantage(r.double().numpy(), group_size)
     np.testing.assert_allclose(a, want, rtol=1e-6, atol=1e-6)
+
+
+@pytest.mark.parametrize("n", [1, 3, 5, 2047, 2049, 9001])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_sizes_and_alignments(n, shift):
+    # whole and partial groups of 4 tokens and blocks of 2,048, several blocks' partial sums; mask
+    # and gradient buffers aligned for the grouped accesses and not; segment bounds inside groups
+    vcs = _vcs()
+    logp, old, ref = _inputs(n, n)
+    rng = np.random.default_rng(n)
+    mask = (rng.random(n) < 0.4).astype(np.uint8)
+    cut = np.unique(np.concatenate([[0, n], rng.integers(0, n + 1, size=min(n, 40))]))
+    cu, st = cut.astype(np.int32), rng.integers(0, 3, size=len(cut) - 1).astype(np.int32)
+    adv = np.array([0.7, -1.1, 0.3], np.float32)
+    m = torch.from_numpy(np.concatenate([np.zeros(shift, np.uint8), mask])).to(DEV)[shift:]
+    dl = torch.full((n + shift,), 9.0, device=DEV)[shift:]
+    loss = torch.empty(1, dtype=torch.float64, device=DEV)
+    nb = vcs.vcs_grpo_loss_workspace_size(n)
+    ws = torch.empty(nb, dtype=torch.uint8, device=DEV)
+    dev = [torch.from_numpy(x).to(DEV) for x in (cu, st, adv)]
+    assert vcs.vcs_grpo_loss(logp.to(DEV), old.to(DEV), ref.to(DEV), m, dev[0], dev[1], len(st), n, dev[2], 3, 0.2,
+                             0.28, 3.0, 1e-4, loss, dl, ws, nb) == 0
+    assert int(ws[:4].view(torch.int32).item()) == 0
+    _tol_check(float(loss.item()), dl.cpu().numpy().astype(np.float64), logp, old, ref, mask, cu, st, adv, 3)

@@ -125,3 +125,35 @@ def test_loss_over_the_stream_fields():
                                  lay["seg_traj"].cpu().numpy(), adv.cpu().numpy(), w.num_traj)
     assert float(loss.item()) == pytest.approx(lo, rel=1e-5, abs=1e-6)
     np.testing.assert_allclose(g.cpu().numpy(), go, rtol=1e-4, atol=1e-7)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 17, 4095, 4096, 4097, 20003])
+@pytest.mark.parametrize("shift", [0, 1, 4])
+def test_sizes_and_alignments(n, shift):
+    # whole and partial groups of 4 and 16 tokens, chunks of 4,096; buffers at 16-byte boundaries
+    # and not (element offset 1: 4 bytes for the words, 1 for the mask)
+    vcs = _vcs()
+    g = torch.Generator().manual_seed(n + shift)
+    gather = torch.randint(0, 500, (n + shift,), generator=g, dtype=torch.int32).to(DEV)[shift:]
+    mask = (torch.randint(0, 3, (n + shift,), generator=g) * 100).to(torch.uint8).to(DEV)[shift:]
+    ids = torch.randint(0, 200000, (500,), generator=g, dtype=torch.int32).to(DEV)
+    lp = -torch.rand(500, generator=g).to(DEV)
+    o_ids = torch.empty(n + shift, dtype=torch.int32, device=DEV)[shift:]
+    o_lp = torch.empty(n + shift, dtype=torch.float32, device=DEV)[shift:]
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    assert vcs.vcs_stream_fields(ids, lp, 500, gather, mask, n, o_ids, o_lp, st) == 0
+    r_ids, r_lp = ostream.stream_fields(ids.cpu().numpy(), lp.cpu().numpy(), gather.cpu().numpy(), mask.cpu().numpy())
+    assert int(st.item()) == 0
+    assert np.array_equal(o_ids.cpu().numpy(), r_ids)
+    assert np.array_equal(o_lp.cpu().numpy().view(np.uint32), r_lp.view(np.uint32))
+    idx = vcs.compact_trainable(mask).cpu().numpy()
+    assert np.array_equal(idx, ostream.compact_trainable(mask.cpu().numpy()))
+
+
+@pytest.mark.parametrize("chunks", [4096, 4097])
+def test_compaction_around_the_scan_launch(chunks):
+    # each block sums the counts before it up to 4,096 chunks; beyond, a launch scans them
+    vcs = _vcs()
+    n = chunks * 4096 - 5
+    mask = (torch.rand(n, generator=torch.Generator(device=DEV).manual_seed(chunks), device=DEV) < 0.1).to(torch.uint8)
+    assert torch.equal(vcs.compact_trainable(mask), mask.nonzero()[:, 0].int())
