@@ -32,6 +32,11 @@ void load_encode_fn() {
     g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
 }
 
+// The workspace header of a call that launches nothing (the first kernel of one that does clears it).
+vcs_status clear_header(void* ws, cudaStream_t st) {
+  return cudaMemsetAsync(ws, 0, kWsHeader, st) == cudaSuccess ? VCS_OK : VCS_ERR_CUDA;
+}
+
 vcs_status check_attn(const AttnArgs& a) {
   if (a.q == nullptr || a.k == nullptr || a.v == nullptr || a.cu_seqlens == nullptr) return VCS_ERR_INVALID_ARG;
   if (a.num_segments < 0 || a.num_tokens < 0 || a.max_seqlen < 0 || a.hq <= 0 || a.hkv <= 0)
@@ -221,8 +226,7 @@ vcs_status vcs_attn_fwd(const void* q, const void* k, const void* v, const int32
     return VCS_ERR_WORKSPACE;
   a.status = static_cast<int32_t*>(ws);
   cudaStream_t st = as_stream(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, st) != cudaSuccess) return VCS_ERR_CUDA;
-  if (num_tokens == 0 || num_segments == 0) return VCS_OK;
+  if (num_tokens == 0 || num_segments == 0) return clear_header(ws, st);
   if (launch_attn_fwd(a, o, lse, ws, st) != cudaSuccess) return VCS_ERR_CUDA;
   return VCS_OK;
 }
@@ -318,8 +322,7 @@ vcs_status vcs_attn_bwd(const void* q, const void* k, const void* v, const void*
     return VCS_ERR_WORKSPACE;
   a.status = static_cast<int32_t*>(ws);
   cudaStream_t st = as_stream(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, st) != cudaSuccess) return VCS_ERR_CUDA;
-  if (num_tokens == 0 || num_segments == 0) return VCS_OK;
+  if (num_tokens == 0 || num_segments == 0) return clear_header(ws, st);
   if (launch_attn_bwd(a, o, lse, dout, dq, dk, dv, ws, st) != cudaSuccess) return VCS_ERR_CUDA;
   return VCS_OK;
 }
@@ -356,8 +359,7 @@ vcs_status vcs_attn_fwd_reuse(const void* q, const void* k, const void* v, const
     return VCS_ERR_WORKSPACE;
   a.status = static_cast<int32_t*>(ws);
   cudaStream_t st = as_stream(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, st) != cudaSuccess) return VCS_ERR_CUDA;
-  if (num_tokens == 0 || num_segments == 0) return VCS_OK;
+  if (num_tokens == 0 || num_segments == 0) return clear_header(ws, st);
   if (launch_attn_fwd(a, o, lse, ws, st) != cudaSuccess) return VCS_ERR_CUDA;
   return VCS_OK;
 }
@@ -392,8 +394,7 @@ vcs_status vcs_attn_fwd_gathered(const void* q_traj, const void* k_traj, const v
     return VCS_ERR_WORKSPACE;
   a.status = static_cast<int32_t*>(ws);
   cudaStream_t st = as_stream(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, st) != cudaSuccess) return VCS_ERR_CUDA;
-  if (num_tokens == 0 || num_segments == 0) return VCS_OK;
+  if (num_tokens == 0 || num_segments == 0) return clear_header(ws, st);
   if (launch_attn_fwd(a, o, lse, ws, st) != cudaSuccess) return VCS_ERR_CUDA;
   return VCS_OK;
 }
@@ -428,8 +429,8 @@ vcs_status vcs_attn_bwd_gathered(const void* q_traj, const void* k_traj, const v
     return VCS_ERR_WORKSPACE;
   a.status = static_cast<int32_t*>(ws);
   cudaStream_t st = as_stream(stream);
-  if (cudaMemsetAsync(ws, 0, kWsHeader, st) != cudaSuccess) return VCS_ERR_CUDA;
   if (num_tokens == 0 || num_segments == 0) {  // no segment token reads the trajectory: zero gradients
+    if (clear_header(ws, st) != VCS_OK) return VCS_ERR_CUDA;
     const size_t qb = (size_t)traj_tokens * hq * d * 2, kb = (size_t)traj_tokens * hkv * d * 2;
     if (traj_tokens > 0 && (cudaMemsetAsync(dq_traj, 0, qb, st) != cudaSuccess ||
                             cudaMemsetAsync(dk_traj, 0, kb, st) != cudaSuccess ||

@@ -44,7 +44,8 @@ template <int D>
 __global__ void __launch_bounds__(kPreThreads) bwd_pre(const __nv_bfloat16* __restrict__ o,
                                                        const __nv_bfloat16* __restrict__ dout, int64_t rows,
                                                        int32_t hq, int64_t num_tokens, float* __restrict__ dvec,
-                                                       float* __restrict__ dq_acc) {
+                                                       float* __restrict__ dq_acc, int32_t* status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = VCS_OK;  // the call's first kernel
   constexpr int CPR = D / 8;  // chunks per row
   const int64_t total = rows * CPR;
   for (int64_t c = blockIdx.x * (int64_t)kPreThreads + threadIdx.x; c - threadIdx.x < total;
@@ -864,7 +865,7 @@ cudaError_t launch_bwd_d(const AttnArgs& a, const void* o, const float* lse, con
     if (blocks > 152 * 32) blocks = 152 * 32;
     bwd_pre<D><<<(unsigned)blocks, kPreThreads, 0, st>>>(static_cast<const __nv_bfloat16*>(o),
                                                          static_cast<const __nv_bfloat16*>(dout), rows, a.hq,
-                                                         a.num_tokens, dvec, GATHER ? nullptr : dq_acc);
+                                                         a.num_tokens, dvec, GATHER ? nullptr : dq_acc, a.status);
   }
   alignas(64) CUtensorMap tq, tk, tv, tdo, tqr, tkr, tvr, tqs, tks, tvs;
   if (GATHER) {

@@ -228,3 +228,14 @@ def test_work_unit_count_on_builder_layouts(window):
     hdr = ws[:256].view(torch.int32).cpu().numpy()
     assert hdr[0] == 0 and hdr[128 // 4] == _units_of(cu, w.hq)
     check_sampled(q, k, v, cu, o, lse, np.random.default_rng(40 + window), n_seg=4, heads=[0, w.hq - 1])
+
+
+@pytest.mark.parametrize("num_segments", [1, 63, 64, 65])
+def test_unit_list_in_one_and_two_launches(num_segments):
+    # up to 64 segments (and 2,048 units) one block scans and lists the units, beyond a second launch
+    # lists them; empty segments among them
+    rng = np.random.default_rng(num_segments)
+    cu = cu_from_lengths([int(x) for x in rng.integers(0, 300, size=num_segments)])
+    q, k, v, _ = workloads.draw_dense(5, max(int(cu[-1]), 1), 2, 1, 64, device="cuda")
+    q, k, v = (x[:int(cu[-1])] for x in (q, k, v))
+    compare_full(q, k, v, cu, *run_fwd(q, k, v, cu))
