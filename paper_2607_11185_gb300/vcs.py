@@ -259,7 +259,25 @@ def _check(status: int, where: str):
 
 
 def _ws(nbytes: int, device) -> torch.Tensor:
-    return torch.empty(max(nbytes, 256), dtype=torch.uint8, device=device)
+    """Workspace of at least nbytes as int32 words; word 0 is the device status of the calls that have one."""
+    return torch.empty((max(nbytes, 256) + 3) // 4, dtype=torch.int32, device=device)
+
+
+def _host_words(n: int, dtype) -> torch.Tensor:
+    """Zeroed pinned host words that kernels write directly: read after _wait, they need neither a fill
+    launch before nor a copy after the call."""
+    t = torch.empty(n, dtype=dtype, pin_memory=True)
+    ctypes.memset(t.data_ptr(), 0, t.numel() * t.element_size())
+    return t
+
+
+def _wait(stream):
+    """Blocks until the work issued so far on the call's stream is done."""
+    if stream is None:
+        stream = torch.cuda.current_stream()
+    elif isinstance(stream, int):
+        stream = torch.cuda.ExternalStream(stream)
+    stream.synchronize()
 
 
 def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stream=None):
@@ -267,16 +285,17 @@ def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stre
     dev = cu_steps.device
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
     nb = vcs_segments_workspace_size(num_traj, num_steps)
-    ws = _ws(nb, dev)
-    sizes = torch.zeros(3, dtype=torch.int64, device=dev)   # 24 bytes = vcs_sizes
+    return _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, _ws(nb, dev), nb, stream)
+
+
+def _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb, stream):
+    sizes = _host_words(3, torch.int64)   # 24 bytes = vcs_sizes
     _check(vcs_plan_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, nb,
                              stream), "vcs_plan_segments")
-    host = sizes.cpu()
-    ns, nt = int(host[0]), int(host[1])
-    mx = int(host[2] & 0xFFFFFFFF)
-    st = int((host[2] >> 32) & 0xFFFFFFFF)
-    _check(st, "vcs_plan_segments (device)")
-    return ns, nt, mx
+    _wait(stream)
+    ns, nt, tail = sizes.tolist()
+    _check(tail >> 32, "vcs_plan_segments (device)")
+    return ns, nt, tail & 0xFFFFFFFF
 
 
 def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, with_mask: bool = True,
@@ -284,10 +303,10 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
     """Plan + build: returns a dict of device tensors and the sizes."""
     dev = cu_steps.device
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
-    ns, nt, mx = plan_segments(cu_steps, step_img, step_txt, window, keep, stream)
     nb = vcs_segments_workspace_size(num_traj, num_steps)
     ws = _ws(nb, dev)
-    sizes = torch.zeros(3, dtype=torch.int64, device=dev)
+    ns, nt, mx = _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb, stream)
+    sizes = _host_words(3, torch.int64)
     out = dict(cu_seqlens=torch.empty(ns + 1, dtype=torch.int32, device=dev),
                seg_traj=torch.empty(ns, dtype=torch.int32, device=dev),
                tok_gather=torch.empty(nt, dtype=torch.int32, device=dev),
@@ -297,8 +316,8 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
     _check(vcs_build_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ns, nt,
                               out["cu_seqlens"], out["seg_traj"], out["tok_gather"], out["tok_src_step"],
                               out["tok_pos"], out["tok_loss_mask"], sizes, ws, nb, stream), "vcs_build_segments")
-    st = int((sizes[2].item() >> 32) & 0xFFFFFFFF)
-    _check(st, "vcs_build_segments (device)")
+    _wait(stream)
+    _check(sizes.tolist()[2] >> 32, "vcs_build_segments (device)")
     out.update(num_segments=ns, num_tokens=nt, max_seqlen=mx)
     return out
 
@@ -311,10 +330,11 @@ def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
     q = torch.empty((nt, hq, d), dtype=q_traj.dtype, device=dev)
     k = torch.empty((nt, hkv, d), dtype=k_traj.dtype, device=dev)
     v = torch.empty((nt, hkv, d), dtype=v_traj.dtype, device=dev)
-    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    status = _host_words(1, torch.int32)
     _check(vcs_gather(q_traj, k_traj, v_traj, q_traj.shape[0], tok_gather, nt, hq, hkv, d, q, k, v, status,
                       stream), "vcs_gather")
-    _check(int(status.item()), "vcs_gather (device)")
+    _wait(stream)
+    _check(status.tolist()[0], "vcs_gather (device)")
     return q, k, v
 
 
@@ -329,7 +349,7 @@ def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, s
     _check(vcs_attn_fwd(q, k, v, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, o, lse, ws, nb,
                         stream), "vcs_attn_fwd")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_attn_fwd (device)")
+        _check(int(ws[0].item()), "vcs_attn_fwd (device)")
     return o, lse
 
 
@@ -344,7 +364,7 @@ def attn_bwd(q, k, v, o, lse, dout, cu_seqlens, max_seqlen: int, softmax_scale: 
     _check(vcs_attn_bwd(q, k, v, o, lse, dout, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, dq, dk,
                         dv, ws, nb, stream), "vcs_attn_bwd")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_attn_bwd (device)")
+        _check(int(ws[0].item()), "vcs_attn_bwd (device)")
     return dq, dk, dv
 
 
@@ -352,10 +372,11 @@ def shared_prefix(cu_seqlens, seg_traj, tok_gather, stream=None):
     """Per segment, its common prefix length with the previous segment of its trajectory."""
     ns = cu_seqlens.numel() - 1
     out = torch.empty(max(ns, 0), dtype=torch.int32, device=cu_seqlens.device)
-    status = torch.zeros(1, dtype=torch.int32, device=cu_seqlens.device)
+    status = _host_words(1, torch.int32)
     _check(vcs_shared_prefix(cu_seqlens, seg_traj, tok_gather, ns, tok_gather.numel(), out, status, stream),
            "vcs_shared_prefix")
-    _check(int(status.item()), "vcs_shared_prefix (device)")
+    _wait(stream)
+    _check(status.tolist()[0], "vcs_shared_prefix (device)")
     return out
 
 
@@ -372,7 +393,7 @@ def attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, max_seqlen: int, softmax_sca
     _check(vcs_attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, o, lse,
                               ws, nb, stream), "vcs_attn_fwd_reuse")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_attn_fwd_reuse (device)")
+        _check(int(ws[0].item()), "vcs_attn_fwd_reuse (device)")
     return o, lse
 
 
@@ -391,7 +412,7 @@ def attn_fwd_gathered(q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen
     _check(vcs_attn_fwd_gathered(q_traj, k_traj, v_traj, tt, tok_gather, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d,
                                  softmax_scale, o, lse, ws, nb, stream), "vcs_attn_fwd_gathered")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_attn_fwd_gathered (device)")
+        _check(int(ws[0].item()), "vcs_attn_fwd_gathered (device)")
     return o, lse
 
 
@@ -410,7 +431,7 @@ def attn_bwd_gathered(q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqle
                                  max_seqlen, hq, hkv, d, softmax_scale, dq, dk, dv, ws, nb, stream),
            "vcs_attn_bwd_gathered")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_attn_bwd_gathered (device)")
+        _check(int(ws[0].item()), "vcs_attn_bwd_gathered (device)")
     return dq, dk, dv
 
 
@@ -428,7 +449,7 @@ def grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv
                          adv.numel(), eps_low, eps_high, clip_cap, kl_coef, loss, dlogp, ws, nb, stream),
            "vcs_grpo_loss")
     if check:
-        _check(int(ws[:4].view(torch.int32).item()), "vcs_grpo_loss (device)")
+        _check(int(ws[0].item()), "vcs_grpo_loss (device)")
     return loss, dlogp
 
 
@@ -438,10 +459,11 @@ def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     dev = tok_gather.device
     ids = torch.empty(nt, dtype=torch.int32, device=dev)
     logp = torch.empty(nt, dtype=torch.float32, device=dev)
-    status = torch.zeros(1, dtype=torch.int32, device=dev)
+    status = _host_words(1, torch.int32)
     _check(vcs_stream_fields(traj_ids, traj_logp, traj_ids.numel(), tok_gather, tok_loss_mask, nt, ids, logp, status,
                              stream), "vcs_stream_fields")
-    _check(int(status.item()), "vcs_stream_fields (device)")
+    _wait(stream)
+    _check(status.tolist()[0], "vcs_stream_fields (device)")
     return ids, logp
 
 
@@ -451,12 +473,13 @@ def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     dev = tok_loss_mask.device
     cap = nt if capacity is None else capacity
     idx = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
-    count = torch.zeros(1, dtype=torch.int64, device=dev)
+    count = _host_words(1, torch.int64)
     nb = vcs_compact_workspace_size(nt)
     ws = _ws(nb, dev)
     _check(vcs_compact_trainable(tok_loss_mask, nt, idx, cap, count, ws, nb, stream), "vcs_compact_trainable")
-    _check(int(ws[:4].view(torch.int32).item()), "vcs_compact_trainable (device)")
-    return idx[: int(count.item())]
+    _check(int(ws[0].item()), "vcs_compact_trainable (device)")
+    _wait(stream)
+    return idx[: count.tolist()[0]]
 
 
 def group_advantage(rewards, group_size: int, eps: float = 1e-6, stream=None):
