@@ -597,7 +597,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool valid = row < L;
         const float inv_l = 1.f / l;
         const uint64_t il2 = f2pack(inv_l, inv_l);
-        __nv_bfloat16* orow = out + ((size_t)(start + row) * hq + h) * D;
+        // The warp's 32 rows pass through its part of the tile's Q buffer (every S of the tile is
+        // complete) so that 8 lanes store a row's 128 bytes: a thread storing its own row in 16-byte
+        // pieces touches 32 lines an instruction, 4,096 cycles of the load/store unit a unit.
+        const uint32_t stage = sbase + (wg == 0 ? C::OFF_Q0 : C::OFF_Q1);
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
@@ -611,12 +614,24 @@ __global__ void __launch_bounds__(kThreads, 1)
             f2unpack(fmul2(f2pack(__uint_as_float(o[2 * e]), __uint_as_float(o[2 * e + 1])), il2), x0, x1);
             pk[e] = pack_bf16(x0, x1);
           }
-          if (valid) {
-            uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
 #pragma unroll
-            for (int v4 = 0; v4 < 4; ++v4) dst[v4] = make_uint4(pk[4 * v4], pk[4 * v4 + 1], pk[4 * v4 + 2], pk[4 * v4 + 3]);
-          }
+          for (int v4 = 0; v4 < 4; ++v4)
+            st_shared_v4(stage + (c / 2) * C::BLOCK + r * 128 + (uint32_t)((((c & 1) * 4 + v4) ^ (r & 7)) << 4),
+                         pk[4 * v4], pk[4 * v4 + 1], pk[4 * v4 + 2], pk[4 * v4 + 3]);
         }
+        asm volatile("" ::: "memory");
+        __syncwarp();
+        asm volatile("" ::: "memory");
+        const int row0 = quad * 32 + (lane >> 3), chunk = lane & 7;
+        __nv_bfloat16* dst = out + ((size_t)(start + mt * C::BM + row0) * hq + h) * D + chunk * 8;
+#pragma unroll
+        for (int kb = 0; kb < C::KB; ++kb)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int ri = row0 + 4 * i;
+            const uint4 v = ld_shared_v4(stage + kb * C::BLOCK + ri * 128 + (uint32_t)((chunk ^ (ri & 7)) << 4));
+            if (mt * C::BM + ri < L) *reinterpret_cast<uint4*>(dst + (size_t)(4 * i) * hq * D + kb * 64) = v;
+          }
         if (valid) lse[(size_t)h * num_tokens + start + row] = (m_run + lg2(l)) * 0.69314718055994531f;
       }
     }
