@@ -684,39 +684,78 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     } else {
       tc_fence_after();
       // warpgroup 1 writes dK, warpgroup 2 writes dV (key row r on the TMEM lane)
-      const int kpos = n * C::BM + r;
       const uint32_t col = k == 0 ? C::TM_DK : C::TM_DV;
-      __nv_bfloat16* outp = (k == 0 ? dk : dv) + ((size_t)(start + kpos) * hkv + g) * D;
-      float* accp = nullptr;  // gathered: fp32 add at the key's trajectory row
-      if (GATHER && kpos < L) {
-        const int t = tok_gather[start + kpos];
-        if (t >= 0 && t < traj_tokens) accp = (k == 0 ? dk_acc : dv_acc) + ((size_t)t * hkv + g) * D;
-      }
+      if constexpr (GATHER) {  // fp32 add at the key's trajectory row
+        const int kpos = n * C::BM + r;
+        float* accp = nullptr;
+        if (kpos < L) {
+          const int t = tok_gather[start + kpos];
+          if (t >= 0 && t < traj_tokens) accp = (k == 0 ? dk_acc : dv_acc) + ((size_t)t * hkv + g) * D;
+        }
 #pragma unroll
-      for (int c = 0; c < D / 32; ++c) {
-        uint32_t v32[32];
-        tmem_ld_32x32b_x32(trow + col + c * 32, v32);
-        tmem_ld_wait();
-        reg_fence<32>(v32);
-        if (GATHER) {
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t v32[32];
+          tmem_ld_32x32b_x32(trow + col + c * 32, v32);
+          tmem_ld_wait();
+          reg_fence<32>(v32);
           if (accp != nullptr) {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
               red_add_v4(accp + c * 32 + e * 4, __uint_as_float(v32[e * 4]), __uint_as_float(v32[e * 4 + 1]),
                          __uint_as_float(v32[e * 4 + 2]), __uint_as_float(v32[e * 4 + 3]));
           }
-        } else if (kpos < L) {
-          uint4* d4 = reinterpret_cast<uint4*>(outp + c * 32);
+        }
+      } else if constexpr (D == 64) {
+        const int kpos = n * C::BM + r;
+        __nv_bfloat16* outp = (k == 0 ? dk : dv) + ((size_t)(start + kpos) * hkv + g) * D;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            uint4 pk;
-            pk.x = pack_bf16(__uint_as_float(v32[q * 8 + 0]), __uint_as_float(v32[q * 8 + 1]));
-            pk.y = pack_bf16(__uint_as_float(v32[q * 8 + 2]), __uint_as_float(v32[q * 8 + 3]));
-            pk.z = pack_bf16(__uint_as_float(v32[q * 8 + 4]), __uint_as_float(v32[q * 8 + 5]));
-            pk.w = pack_bf16(__uint_as_float(v32[q * 8 + 6]), __uint_as_float(v32[q * 8 + 7]));
-            d4[q] = pk;
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t v32[32];
+          tmem_ld_32x32b_x32(trow + col + c * 32, v32);
+          tmem_ld_wait();
+          reg_fence<32>(v32);
+          if (kpos < L) {
+            uint4* d4 = reinterpret_cast<uint4*>(outp + c * 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              d4[q] = make_uint4(pack_bf16(__uint_as_float(v32[q * 8 + 0]), __uint_as_float(v32[q * 8 + 1])),
+                                 pack_bf16(__uint_as_float(v32[q * 8 + 2]), __uint_as_float(v32[q * 8 + 3])),
+                                 pack_bf16(__uint_as_float(v32[q * 8 + 4]), __uint_as_float(v32[q * 8 + 5])),
+                                 pack_bf16(__uint_as_float(v32[q * 8 + 6]), __uint_as_float(v32[q * 8 + 7])));
           }
         }
+      } else {
+        // the warp's 32 rows pass through its part of the K or V buffer (every MMA is complete), so
+        // that 8 lanes store a row's 128 bytes instead of a thread its own row in 16-byte pieces (8
+        // short rollouts 6.88 -> 6.75 ms, 32 segments of 1,024 0.327 -> 0.304; at d = 64 it cost 1%)
+        const uint32_t stage = sbase + (k == 0 ? C::OFF_K : C::OFF_V);
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t v32[32];
+          tmem_ld_32x32b_x32(trow + col + c * 32, v32);
+          tmem_ld_wait();
+          reg_fence<32>(v32);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            st_shared_v4(stage + (c / 2) * C::BLOCK + r * 128 + (uint32_t)((((c & 1) * 4 + q) ^ (r & 7)) << 4),
+                         pack_bf16(__uint_as_float(v32[q * 8 + 0]), __uint_as_float(v32[q * 8 + 1])),
+                         pack_bf16(__uint_as_float(v32[q * 8 + 2]), __uint_as_float(v32[q * 8 + 3])),
+                         pack_bf16(__uint_as_float(v32[q * 8 + 4]), __uint_as_float(v32[q * 8 + 5])),
+                         pack_bf16(__uint_as_float(v32[q * 8 + 6]), __uint_as_float(v32[q * 8 + 7])));
+        }
+        asm volatile("" ::: "memory");
+        __syncwarp();
+        asm volatile("" ::: "memory");
+        const int row0 = quad * 32 + (lane >> 3), chunk = lane & 7;
+        __nv_bfloat16* dst = (k == 0 ? dk : dv) + ((size_t)(start + n * C::BM + row0) * hkv + g) * D + chunk * 8;
+#pragma unroll
+        for (int kb = 0; kb < C::KB; ++kb)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int ri = row0 + 4 * i;
+            const uint4 v = ld_shared_v4(stage + kb * C::BLOCK + ri * 128 + (uint32_t)((chunk ^ (ri & 7)) << 4));
+            if (n * C::BM + ri < L) *reinterpret_cast<uint4*>(dst + (size_t)(4 * i) * hkv * D + kb * 64) = v;
+          }
       }
     }
   } else {
