@@ -102,26 +102,33 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 //   S^T(u) -> P^T(u) (compute warps) -> dV += P^T dO
 //   dP^T(u) -> dS^T(u) (compute warps) -> dK += dS^T Q, dQ(u) -> drain
 // Two warps issue MMAs, one for each chain, so that a barrier wait of one (about 250 cycles while the
-// pipe streams from shared memory) is covered by the other's MMAs.  The order on the pipe is dP^T(u),
-// dV(u), S^T(u+1), dK(u), dQ(u): dP^T(u) follows the drain's read of dQ(u-1) (d = 128: it overwrites
-// its columns), dV(u) and S^T(u+1) run while dS^T(u) is computed, and
-// P^T(u+1) is computed while dK(u), dQ(u) and that read run.
+// pipe streams from shared memory) is covered by the other's MMAs.
+// d = 128: the order on the pipe is dP^T(u), dV(u), S^T(u+1), dK(u), dQ(u): dP^T(u) follows the
+// drain's read of dQ(u-1), whose columns it overwrites, dV(u) and S^T(u+1) run while dS^T(u) is
+// computed, and P^T(u+1) is computed while dK(u), dQ(u) and that read run.
 // What bounds it is the shared-memory pipe: per tile at d = 128 the MMAs read 256 KB (2,048 cycles
 // at 128 B/clk), TMA writes 64 KB (512), dS^T and the row terms take 512 and the dQ reductions about
 // 990 (measured against a stream of shared loads).  Before, S^T and dP^T were issued together, one
 // pass of the compute warps made P^T and dS^T of both, and dQ left through shared memory by TMA
 // reduce-adds, whose engine also carries the tile loads (64 KB at 25.5 B/clk + 64 KB at 37 B/clk).
-// vcs_attn_bwd, 40/8/128, four segments of 8,192: 6.18 ms before, 5.34 now (892 -> 1,030 TFLOP/s
-// credited); 14/2/64, sixteen of 4,096, where the kernel before was a serial loop with 16-byte
-// reductions of 32 different rows: 3.89 -> 1.52 ms (247 -> 633).
+// vcs_attn_bwd, 40/8/128, four segments of 8,192: 6.18 ms before, 5.31 now (892 -> 1,035 TFLOP/s
+// credited).
+// d = 64: the MMAs need about 1,400 cycles a tile; the compute warps' two passes (about 1,000 and
+// 1,100, mostly latencies of one warp's chain: neither leaving out the reductions nor the stores of
+// dS^T shortens them) bound it, so everything they wait for is issued a step ahead: TMEM has room
+// for dQ and P^T in columns of their own, so S^T(u+1) is issued when S^T(u) has been read, not when
+// dV(u) has, and dP^T(u+1) right behind dK(u), not behind the drain's read.  14/2/64, sixteen of
+// 4,096: 3.89 ms for the serial loop with 16-byte reductions of 32 different rows that was here
+// first, 1.42 for the order of d = 128, 1.35 with dP^T ahead, 1.29 with S^T ahead too, 1.27 with the
+// drain's pace set again (247 -> 759 TFLOP/s credited).
 //   WG0   warp 0: TMA producer (K and V once, NST tiles of Q and dO in flight)
-//         warp 1: TMEM allocation, MMAs of S^T and dV;  warp 2: MMAs of dP^T, dK and dQ
+//         warp 1: TMEM allocation, MMAs of S^T and dV;  warp 2: MMAs of dP^T, dK and dQ;  warp 3: row terms
 //         (both run warp-uniformly up to an elected lane's issue, which keeps descriptors in uniform
 //         registers: 7.6 -> 6.7 ms on the case above while it was being built)
 //   WG1/2 compute: warpgroup k takes query columns [64k, 64k+64), a thread one key row.  P^T stays
-//         in fp32 registers between its two passes; its bf16 copy goes over the S^T columns the
-//         thread has read (the A operand of dV += P^T dO), dS^T over its dP^T columns (A of
-//         dK += dS^T Q) and to shared memory (for dQ)
+//         in fp32 registers between its two passes; its bf16 copy goes to TMEM (the A operand of
+//         dV += P^T dO), dS^T over the dP^T columns the thread has read (A of dK += dS^T Q) and to
+//         shared memory (for dQ)
 //   WG3   dQ drain: TMEM -> registers -> fp32 reductions into the accumulator.  An SM sends 32 B a
 //         clock to L2 and a 128-byte line costs a fifth flit, so 25.5 B/clk (2,570 cycles for
 //         64 KB) is the ceiling for TMA bulk reduce-adds and register reductions alike, if a warp's
@@ -130,8 +137,9 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 //         dims of one query and a scalar reduction is one line.  d = 64 (M = 64 would halve the
 //         rate): dQ = dS^T K, and two rounds of lane exchanges make 8 lanes hold a 128-byte row
 //         piece.
-// TMEM (512 columns): dV, dK (D each), S^T/P^T (128), dP^T/dS^T (128); dQ goes over the dP^T
-// columns at d = 128 (dK(u) reads dS^T there first, in pipe order) and has its own at d = 64.
+// TMEM (512 columns): dV, dK (D each), S^T (128), dP^T/dS^T (128).  d = 128: P^T goes over the S^T
+// columns and dQ over the dP^T columns (dK(u) reads dS^T there first, in pipe order).  d = 64: dQ
+// and P^T have 64 columns each.
 
 // TMEM loads / stores of N consecutive 32-bit columns of the warp's 32 lanes.
 template <int N>
@@ -158,17 +166,25 @@ struct Bwd {
   static constexpr int OFF_V = TILE;
   static constexpr int OFF_QD = 2 * TILE;
   static constexpr int OFF_DS = OFF_QD + 2 * NST * TILE;  // dS^T [128 keys][128 queries], two 64-query blocks
-  static constexpr int OFF_ROW = OFF_DS + 2 * BLOCK;  // [tile parity][WG k]: -lse*log2e of 64 queries, then -D*scale
+  static constexpr int NDS = D == 128 ? 1 : 2;              // buffers of dS^T, by tile parity
+  static constexpr int OFF_ROW = OFF_DS + NDS * 2 * BLOCK;  // [tile parity][WG k]: -lse*log2e of 64 queries, -D*scale
   static constexpr int OFF_BAR = OFF_ROW + 2 * 2 * 128 * 4;
   static constexpr int BAR_BYTES = 512;
   static constexpr int SMEM = OFF_BAR + BAR_BYTES;
   static constexpr int TM_DV = 0, TM_DK = D, TM_S = 2 * D, TM_P = 2 * D + 128;
   static constexpr bool OWN_DQ = D == 64;
   static constexpr int TM_DQ = OWN_DQ ? TM_P + 128 : TM_P;
-  // P^T and dS^T of queries [16kk, 16kk+16): 8 columns of bf16 pairs at this offset of TM_S / TM_P
-  // (each warpgroup's 64 columns hold its 32 words a row at their start)
-  __host__ __device__ static constexpr uint32_t pt_col(int kk) { return 64 * (kk >> 2) + 8 * (kk & 3); }
-  static constexpr int REG_CTRL = 80, REG_COMPUTE = 144, REG_DRAIN = 144;
+  static constexpr bool OWN_PT = D == 64;
+  static constexpr int TM_PT = OWN_PT ? TM_DQ + 64 : TM_S;
+  static constexpr int PT_WG = OWN_PT ? 32 : 64;  // columns from one warpgroup's P^T to the next's
+  // queries [16kk, 16kk+16) of P^T / dS^T: 8 columns of bf16 pairs (each warpgroup's 32 words a row
+  // are at the start of its 64 columns, or alone in P^T's own)
+  __host__ __device__ static constexpr uint32_t pt_col(int kk) { return TM_PT + PT_WG * (kk >> 2) + 8 * (kk & 3); }
+  __host__ __device__ static constexpr uint32_t ds_col(int kk) { return TM_P + 64 * (kk >> 2) + 8 * (kk & 3); }
+  // Row terms staged by warp 3, or by the compute warps.  d = 64, which the compute warps bound: 1.34
+  // ms against 1.29 (14/2/64, sixteen segments of 4,096); d = 128: 0.5% slower by a warp of its own.
+  static constexpr bool ROW_WARP = D == 64;
+  static constexpr int REG_CTRL = ROW_WARP ? 96 : 80, REG_COMPUTE = ROW_WARP ? 136 : 144, REG_DRAIN = 144;
   static constexpr int REG_LAUNCH = 65536 / THREADS;
   // Tile u's Q and dO take the slots 2(u % NST) and the next, in turn: dO(u) is released well
   // before Q(u), and S^T needs Q(u+NST) before dV and dP^T need dO(u+NST), so Q(u+NST) goes where
@@ -188,7 +204,9 @@ struct BwdBars {
   uint64_t kv_full;
   uint64_t q_full[4], q_done[4];     // Q(u) landed; its last reader dK(u) complete
   uint64_t do_full[4], do_done[4];   // dO(u) landed; its readers dV(u) and dP^T(u) complete
-  uint64_t s_full;                   // S^T(u) complete
+  uint64_t s_full;                   // S^T(u) complete (ROW_WARP: and its row terms staged)
+  uint64_t rt_free[2];               // ROW_WARP: the row terms of the tile of this parity no longer needed
+  uint64_t s_read;                   // d = 64: S^T(u) read out of TMEM
   uint64_t p_full;                   // P^T(u) written, dP^T(u) issued (so that dV(u) does not run ahead of it)
   uint64_t dp_full;                  // dP^T(u) complete
   uint64_t ds_full[2];               // dS^T(u): columns [0,32) / [32,64) of each warpgroup written
@@ -205,7 +223,8 @@ static_assert(sizeof(BwdBars) <= Bwd<64>::BAR_BYTES && sizeof(BwdBars) <= Bwd<12
 // exchange with lane^1 makes 4 consecutive columns of 64-byte row pieces, one with lane^4 makes
 // 128-byte pieces: 8 lanes a row, 4 rows a reduction.  row(i, live) gives the accumulator row of the
 // warp's query i and whether its values are added (else 0 is).  Four reductions (16 lines of 128
-// bytes) a warp every 400 cycles: 1.52 ms against 1.65 at full speed (14/2/64, 16 segments of 4,096).
+// bytes) a warp every 200 cycles: 1.268 ms (14/2/64, 16 segments of 4,096) against 1.293 at full
+// speed and 1.273 and 1.288 with 300 and 400.
 template <typename RowFn>
 __device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, RowFn row) {
   const bool odd = lane & 1, oddr = lane & 4;
@@ -245,7 +264,7 @@ __device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, 
         red_add_v4(po + 32 * i + coff, o[0], o[1], o[2], o[3]);
       }
       if (g == 0 || half == 0)
-        while ((uint32_t)clock() - t0 < (uint32_t)(400 * (2 * g + half + 1))) {
+        while ((uint32_t)clock() - t0 < (uint32_t)(200 * (2 * g + half + 1))) {
         }
     }
 }
@@ -321,6 +340,17 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     }
   };
   const Walk walk0{nsub - 1, g * G, g * G, G};
+  // lse and D of query i of w's tile, as loaded: scaled only where they are staged
+  auto row_terms = [&](const Walk& w, int i, bool mine, float& l, float& dd) {
+    l = __int_as_float(0x7f800000);  // +inf: query outside the segment -> P = 0
+    dd = 0.f;
+    const int q = n * C::BM + w.sub * C::BQ + i;
+    if (w.sub >= 0 && mine && q < L) {
+      const size_t j = (size_t)w.head * num_tokens + start + q;
+      l = __ldg(&lse[j]);
+      dd = __ldg(&dvec[j]);
+    }
+  };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sbase = smem_u32(smem);
@@ -333,7 +363,9 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       mbar_init(&bars->do_full[i], 1);
       mbar_init(&bars->do_done[i], 2);
     }
-    mbar_init(&bars->s_full, 1);
+    mbar_init(&bars->s_full, C::ROW_WARP ? 2 : 1);
+    for (int i = 0; i < 2; ++i) mbar_init(&bars->rt_free[i], 8);
+    mbar_init(&bars->s_read, 8);
     mbar_init(&bars->p_full, 256 + 1);
     mbar_init(&bars->dp_full, 1);
     for (int i = 0; i < 2; ++i) mbar_init(&bars->ds_full[i], 256);
@@ -452,19 +484,26 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       };
       bool ok = mbar_wait(&bars->kv_full, 0);
       if (warp == 1) {
-        // S^T and dV.  S^T(u+1) overwrites P^T(u), which dV(u), issued before, reads first.
+        // S^T and dV.  d = 128: S^T(u+1) overwrites P^T(u), which dV(u), issued before, reads first.
+        // d = 64: P^T has columns of its own, so S^T(u+1) is issued as soon as S^T(u) is read; its
+        // barrier is then completed by dV(u), which also frees P^T's columns.
         auto issue_s = [&](int u) -> bool {
           if (!mbar_wait(&bars->q_full[u % C::NST], (u / C::NST) & 1)) return false;
+          if (C::OWN_PT && u > 0 && !mbar_wait(&bars->s_read, (u - 1) & 1)) return false;
           tc_fence_after();
           if (elect_one()) {
             issue_kmaj(tmem + C::TM_S, k_kmaj, desc_at(qd_kmaj, C::q_off(u)));
-            tc_commit(&bars->s_full);
+            if (!C::OWN_PT || u == 0) tc_commit(&bars->s_full);
           }
           __syncwarp();
           return true;
         };
         ok = ok && issue_s(0);
         for (int u = 0; ok && u < U; ++u) {
+          if (C::OWN_PT && u + 1 < U && !issue_s(u + 1)) {
+            ok = false;
+            break;
+          }
           if (!mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1) || !mbar_wait(&bars->p_full, u & 1) ||
               aborted_now()) {
             ok = false;
@@ -475,24 +514,25 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
             const uint64_t dmn = desc_at(qd_mnmaj, C::do_off(u));
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              tc_mma_ts(tmem + C::TM_DV, tmem + C::TM_S + C::pt_col(kk), desc_at(dmn, kk * 2048), C::IDESC_KV,
+              tc_mma_ts(tmem + C::TM_DV, tmem + C::pt_col(kk), desc_at(dmn, kk * 2048), C::IDESC_KV,
                         (u > 0 || kk > 0) ? 1u : 0u);
             tc_commit(&bars->do_done[u % C::NST]);
+            if (C::OWN_PT && u + 1 < U) tc_commit(&bars->s_full);
           }
           __syncwarp();
-          if (u + 1 < U) ok = issue_s(u + 1);
+          if (!C::OWN_PT && u + 1 < U) ok = issue_s(u + 1);
         }
       } else {
         // dP^T, dK and dQ.  d = 128: dP^T(u) goes where dQ(u-1) was, dQ(u) where dS^T(u) was, which
-        // dK(u), issued before, reads first; d = 64: dQ(u) goes where dQ(u-1) was.
+        // dK(u), issued before, reads first.  d = 64: dQ(u) goes where dQ(u-1) was, in columns of its
+        // own, so dP^T(u+1) need not wait for it and is issued ahead (what the compute warps wait for
+        // next); dS^T in shared memory then takes two buffers.
         const uint64_t v_kmaj = desc_at(k_kmaj, C::OFF_V);
         const uint64_t ds_mnmaj = desc_at(k_mnmaj, C::OFF_DS);
-        for (int u = 0; ok && u < U; ++u) {
+        auto issue_dp = [&](int u) -> bool {
           if (!mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1) ||
-              (!C::OWN_DQ && u > 0 && !mbar_wait(&bars->dq_free, (u - 1) & 1)) || aborted_now()) {
-            ok = false;
-            break;
-          }
+              (!C::OWN_DQ && u > 0 && !mbar_wait(&bars->dq_free, (u - 1) & 1)) || aborted_now())
+            return false;
           tc_fence_after();
           if (elect_one()) {
             issue_kmaj(tmem + C::TM_P, v_kmaj, desc_at(qd_kmaj, C::do_off(u)));
@@ -501,6 +541,14 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
             tc_commit(&bars->do_done[u % C::NST]);
           }
           __syncwarp();
+          return true;
+        };
+        if (C::OWN_DQ) ok = ok && issue_dp(0);
+        for (int u = 0; ok && u < U; ++u) {
+          if (!C::OWN_DQ && !issue_dp(u)) {
+            ok = false;
+            break;
+          }
           const uint64_t qmn = desc_at(qd_mnmaj, C::q_off(u));
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
@@ -511,22 +559,24 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
                 const int kk = 4 * (j >> 1) + 2 * hf + (j & 1);
-                tc_mma_ts(tmem + C::TM_DK, tmem + C::TM_P + C::pt_col(kk), desc_at(qmn, kk * 2048), C::IDESC_KV,
+                tc_mma_ts(tmem + C::TM_DK, tmem + C::ds_col(kk), desc_at(qmn, kk * 2048), C::IDESC_KV,
                           (u > 0 || hf > 0 || j > 0) ? 1u : 0u);
               }
             }
             __syncwarp();
           }
-          if (ok && C::OWN_DQ && u > 0) {
-            ok = mbar_wait(&bars->dq_free, (u - 1) & 1);
+          if (C::OWN_DQ) {
+            if (ok && u + 1 < U) ok = issue_dp(u + 1);
+            if (ok && u > 0) ok = mbar_wait(&bars->dq_free, (u - 1) & 1);
             tc_fence_after();
           }
           if (!ok) break;
           if (elect_one()) {
+            const uint64_t ds = desc_at(ds_mnmaj, (u % C::NDS) * 2 * C::BLOCK);
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
-              tc_mma_ss(tmem + C::TM_DQ, desc_at(D == 128 ? k_mnmaj : ds_mnmaj, kk * 2048),
-                        desc_at(D == 128 ? ds_mnmaj : k_mnmaj, kk * 2048), C::IDESC_DQ, kk > 0 ? 1u : 0u);
+              tc_mma_ss(tmem + C::TM_DQ, desc_at(D == 128 ? k_mnmaj : ds, kk * 2048),
+                        desc_at(D == 128 ? ds : k_mnmaj, kk * 2048), C::IDESC_DQ, kk > 0 ? 1u : 0u);
             tc_commit(&bars->dq_full);
           }
           __syncwarp();
@@ -535,6 +585,37 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       if (elect_one()) tc_commit(&bars->acc_done);
       __syncwarp();
       if (!ok) abort_now();
+    } else if (C::ROW_WARP && warp == 3) {
+      // ---------------------------------------------------------- row terms
+      // Stages -lse*log2e and -D*scale of each tile's 128 queries for the compute warps, loaded a tile
+      // ahead (behind the drain's reductions a load can take more than a tile's time), and joins S^T's
+      // barrier, so that the compute warps wait once for both.
+      Walk w = walk0;
+      float l[4], dd[4];
+      auto load = [&]() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) row_terms(w, 32 * i + lane, true, l[i], dd[i]);
+        w.next();
+      };
+      load();
+      bool ok = true;
+      float* rows = reinterpret_cast<float*>(smem + C::OFF_ROW);
+      for (int u = 0; u < U; ++u) {
+        if (u >= 2 && !mbar_wait_warp(&bars->rt_free[u & 1], ((u >> 1) - 1) & 1)) { ok = false; break; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // warpgroup i/2's 64 queries: nl, then nd
+          float* r = rows + (u & 1) * 256 + (i >> 1) * 128 + (i & 1) * 32 + lane;
+          r[0] = -l[i] * 1.4426950408889634f;
+          r[64] = -dd[i] * scale;
+        }
+        load();
+        __syncwarp();
+        // S^T(u-1) has completed the phase before
+        if (u > 0 && !mbar_wait_warp(&bars->s_full, (u - 1) & 1)) { ok = false; break; }
+        if (lane == 0) mbar_arrive(&bars->s_full);
+        if (__any_sync(0xffffffffu, aborted_now())) break;
+      }
+      if (!ok) abort_now();
     }
   } else if (warp < 12) {
     // ------------------------------------------------------------ compute
@@ -542,55 +623,59 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     const int k = (warp - 4) >> 2;   // query columns [64k, 64k+64) of the tile
     const int quad = warp & 3;
     const int r = quad * 32 + lane;  // TMEM lane: key row
-    const int tw = threadIdx.x - 128 - k * 128;
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
     // row terms of the warpgroup's 64 queries: nl = -lse*log2e, then nd = -D*scale; two buffers
-    float* rt_s = reinterpret_cast<float*>(smem + C::OFF_ROW) + k * 128;
-    const uint32_t rt_u32 = smem_u32(rt_s);
+    const uint32_t rt_u32 = smem_u32(smem + C::OFF_ROW) + k * 512;
     const uint32_t ds_row = sbase + C::OFF_DS + k * C::BLOCK + r * 128;
     const uint64_t sl2 = f2pack(scale_log2, scale_log2), sc2 = f2pack(scale, scale);
-    // lse and D as loaded, two tiles ahead (behind the drain's reductions a load can take more than
-    // a tile's time); scaled only where they are staged
-    Walk wr = walk0, wc = walk0;  // of the next row terms to load, of the tile computed
-    auto row_terms = [&](float& l, float& dd) {
-      l = __int_as_float(0x7f800000);  // +inf: query outside the segment -> P = 0
-      dd = 0.f;
-      const int q = n * C::BM + wr.sub * C::BQ + 64 * k + tw;
-      if (wr.sub >= 0 && tw < 64 && q < L) {
-        const size_t i = (size_t)wr.head * num_tokens + start + q;
-        l = __ldg(&lse[i]);
-        dd = __ldg(&dvec[i]);
-      }
+    Walk wc = walk0;  // of the tile computed
+    bool ok = true;
+    // without a warp for them: the row terms of the warpgroup's queries, loaded two tiles ahead
+    const int tw = threadIdx.x - 128 - k * 128;
+    float* rt_s = reinterpret_cast<float*>(smem + C::OFF_ROW) + k * 128;
+    Walk wr = walk0;
+    float l0, d0, l1, d1;
+    auto next_terms = [&](float& l, float& dd) {
+      row_terms(wr, 64 * k + tw, tw < 64, l, dd);
       wr.next();
     };
-    float l0, d0, l1, d1;
-    row_terms(l0, d0);
-    row_terms(l1, d1);
-    bool ok = true, got = true;
+    if constexpr (!C::ROW_WARP) {
+      next_terms(l0, d0);
+      next_terms(l1, d1);
+    }
     for (int u = 0; u < U; ++u) {
       // the query rows are the key tile's own: mask keys after queries (column c of the
       // warpgroup is hidden from key row r when c < dlim)
       const int dlim = wc.sub == 0 ? r - 64 * k : 0;
       wc.next();
       const uint32_t rt = rt_u32 + (u & 1) * 1024;
-      if (tw < 64) {
-        rt_s[(u & 1) * 256 + tw] = -l0 * 1.4426950408889634f;
-        rt_s[(u & 1) * 256 + 64 + tw] = -d0 * scale;
+      if constexpr (!C::ROW_WARP) {
+        if (tw < 64) {
+          rt_s[(u & 1) * 256 + tw] = -l0 * 1.4426950408889634f;
+          rt_s[(u & 1) * 256 + 64 + tw] = -d0 * scale;
+        }
+        l0 = l1;
+        d0 = d1;
+        next_terms(l1, d1);
+        // the row terms are staged and everyone is done with the other buffer's; go on only if every
+        // thread got the tile before and no other role has given up
+        if (!named_bar_and(1 + k, 128, ok && !aborted_now())) { ok = false; break; }
       }
-      l0 = l1;
-      d0 = d1;
-      row_terms(l1, d1);
-      // the row terms are staged and everyone is done with the other buffer's; go on only if every
-      // thread got the tile before and no other role has given up
-      if (!named_bar_and(1 + k, 128, got && !aborted_now())) { ok = false; break; }
       uint4 rq[2][4];  // the row terms of 16 columns, and of the next 16
+      auto first_terms = [&](uint32_t at) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) rq[0][j] = ld_shared_v4(rt + 16 * j);
-      // each wait's outcome is the warp's (the TMEM loads below are warp-collective); the
-      // warpgroup decides together at the barrier that opens the next tile
-      got = mbar_wait_warp(&bars->s_full, u & 1);
-      if (!got) continue;
+        for (int j = 0; j < 4; ++j) rq[0][j] = ld_shared_v4(at + 16 * j);
+      };
+      if (!C::ROW_WARP) first_terms(rt);
+      // each wait's outcome is the warp's (the TMEM loads below are warp-collective); without ROW_WARP
+      // the warpgroup decides together at the barrier that opens the next tile
+      if (!mbar_wait_warp(&bars->s_full, u & 1)) {
+        ok = false;
+        if (C::ROW_WARP) break;
+        continue;
+      }
       tc_fence_after();
+      if (C::ROW_WARP) first_terms(rt);
       // P^T = 2^(S^T * scale*log2e - lse*log2e), fp32 in p, bf16 over the S^T columns just read
       uint32_t p[2][32];
       tmem_ld_cols<32>(trow + C::TM_S + 64 * k, p[0]);
@@ -598,6 +683,11 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       tmem_ld_wait();
       reg_fence<32>(p[0]);
       reg_fence<32>(p[1]);
+      if constexpr (C::OWN_PT) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->s_read);
+      }
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
         if (ch < 3) {
@@ -625,15 +715,17 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
 #pragma unroll
         for (int c2 = 0; c2 < 8; ++c2)
           pk[c2] = pack_bf16(__uint_as_float(x[x0 + 2 * c2]), __uint_as_float(x[x0 + 2 * c2 + 1]));
-        tmem_st_32x32b_x8(trow + C::TM_S + 64 * k + 8 * ch, pk);
+        tmem_st_32x32b_x8(trow + C::TM_PT + C::PT_WG * k + 8 * ch, pk);
       }
       tmem_st_wait();
       tc_fence_before();
       mbar_arrive(&bars->p_full);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) rq[0][j] = ld_shared_v4(rt + 256 + 16 * j);
-      got = mbar_wait_warp(&bars->dp_full, u & 1);
-      if (!got) continue;
+      first_terms(rt + 256);
+      if (!mbar_wait_warp(&bars->dp_full, u & 1)) {
+        ok = false;
+        if (C::ROW_WARP) break;
+        continue;
+      }
       tc_fence_after();
       // dS^T = P^T (dP^T - D) * scale, 16 columns at a time, the next ones' loads in flight
       uint32_t dp[2][16];
@@ -662,8 +754,8 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-          st_shared_v4(ds_row + (uint32_t)(((2 * ch + j) ^ (r & 7)) << 4), wd[4 * j], wd[4 * j + 1], wd[4 * j + 2],
-                       wd[4 * j + 3]);
+          st_shared_v4(ds_row + (u % C::NDS) * 2 * C::BLOCK + (uint32_t)(((2 * ch + j) ^ (r & 7)) << 4),
+                       wd[4 * j], wd[4 * j + 1], wd[4 * j + 2], wd[4 * j + 3]);
         tmem_st_32x32b_x8(trow + C::TM_P + 64 * k + 8 * ch, wd);
         if (ch & 1) {
           fence_proxy_async_smem();
@@ -676,8 +768,11 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           reg_fence<16>(dp[cur ^ 1]);
         }
       }
+      if constexpr (C::ROW_WARP) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->rt_free[u & 1]);
+      }
     }
-    ok = ok && got;
     if (ok) ok = mbar_wait_warp(&bars->acc_done, 0);
     if (!ok) {
       abort_now();
