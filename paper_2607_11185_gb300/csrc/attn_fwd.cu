@@ -24,18 +24,20 @@
 // grid is an upper bound of the count, and the few CTAs past it exit at once.
 //
 // Warp roles (384 threads):
-//   warp 0      TMA producer: Q0/Q1 once, then K and V tiles into a 5-slot ring
-//               (K runs one tile ahead of V: K0, K1, V0, K2, V1, ...)
-//   warp 1      TMEM allocator and single-thread tcgen05.mma issuer
-//   warps 2-3   idle (they keep the softmax warps on TMEM lane quadrants 0-3)
+//   warp 0      TMA producer: Q0/Q1 once, then K and V tiles into a ring of 5 slots
+//               (8 at d = 64; K runs one tile ahead of V: K0, K1, V0, K2, V1, ...)
+//   warp 1      TMEM allocator and tcgen05.mma issuer (an elected lane); at d = 64 of S only
+//   warp 2      d = 64: issuer of P V
+//   warp 3      (and 2 at d = 128) idle: they keep the softmax warps on TMEM lane quadrants 0-3
 //   warps 4-7   softmax + epilogue for tile 0 (thread = query row)
 //   warps 8-11  softmax + epilogue for tile 1
 // TMEM (512 columns x 128 lanes, fp32): S0 [0,128), S1 [128,256),
-// O0 [256,256+D), O1 [384,384+D).  P_k (bf16, two per column) overwrites the
-// first 64 columns of S_k and is the A operand of O_k += P_k V read straight
-// from TMEM, so P never touches shared memory.
+// O0 [256,256+D), O1 [384,384+D).  P_k (bf16, two per column) is the A operand of
+// O_k += P_k V read straight from TMEM, so P never touches shared memory.
+// d = 128: P_k overwrites the first 64 columns of S_k.  d = 64 leaves it columns of
+// its own, after O_k.
 //
-// Per K/V tile j the MMA thread issues, for each tile k once its P_k(j) is in
+// d = 128: per K/V tile j the MMA warp issues, for each tile k once its P_k(j) is in
 // TMEM: O_k += P_k(j) V_j, then S_k(j+1) = Q_k K_{j+1}^T.  The tensor pipe
 // executes in order, so the completion of S_k(j+1) also means that P_k(j) has
 // been consumed and O_k is up to date, which is all the softmax warps wait
@@ -49,6 +51,13 @@
 // the two tiles step j reads, K_{j+1} and V_j, next to each other, so the
 // tiled loads complete one barrier per step and the MMA thread waits once a
 // step for its K/V, at the top of the step.
+//
+// d = 64: the MMAs of a step take about 1,020 cycles and the softmax warps bound it, so
+// S_k(j+1) is issued as soon as S_k(j) is in their registers and is complete when they come
+// back for it; before they store P_k(j) they wait for P_k(j-1) V.  One warp issues S and one P V,
+// each waiting for its own ring items.  14/2/64, sixteen segments of 4,096: 0.554 -> 0.523 ms
+// (869 -> 919 TFLOP/s; about 2,100 cycles a step, of which the exponentials of both tiles take
+// 1,024 at 32 a clock).
 //
 // Online softmax with a lazy running maximum: the row maximum used for P is
 // only raised (and O, l rescaled) when a new tile's maximum exceeds it by more
@@ -79,7 +88,8 @@ struct Fwd {
   static constexpr int KB = D / 64;                 // 128-byte column blocks per row
   static constexpr int TILE = BM * D * 2;           // bytes of a 128 x D bf16 tile
   static constexpr int BLOCK = BM * 128;            // bytes of one 128 x 64 column block
-  static constexpr int NSLOT = 5;
+  static constexpr bool OWN_P = D == 64;            // P in TMEM columns of its own
+  static constexpr int NSLOT = OWN_P ? 8 : 5;
   static constexpr int NGRP = 4;                    // ring-item group barriers (tiled loads)
   static constexpr int OFF_Q0 = 0;
   static constexpr int OFF_Q1 = TILE;
@@ -87,6 +97,7 @@ struct Fwd {
   static constexpr int OFF_BAR = OFF_KV + NSLOT * TILE;
   static constexpr int SMEM = OFF_BAR + 256 + 1024;
   static constexpr int TM_S0 = 0, TM_S1 = 128, TM_O0 = 256, TM_O1 = 384;
+  static constexpr int TM_P0 = OWN_P ? TM_O0 + 64 : TM_S0, TM_P1 = OWN_P ? TM_O1 + 64 : TM_S1;
   static constexpr uint32_t IDESC_S = idesc_bf16(128, 128, 0, 0);   // Q (K-major) x K^T (K-major)
   static constexpr uint32_t IDESC_PV = idesc_bf16(128, D, 0, 1);    // P (TMEM) x V (MN-major)
 };
@@ -94,15 +105,18 @@ static_assert(Fwd<128>::SMEM <= 232448, "shared memory budget");
 
 struct Bars {
   uint64_t q_full;
-  uint64_t kv_full[5];   // per ring slot (gathered loads)
-  uint64_t kv_empty[5];
-  uint64_t grp_full[4];  // per pair of ring items consumed in one step (tiled loads)
+  uint64_t kv_full[8];   // per ring slot (gathered loads, OWN_P)
+  uint64_t kv_empty[8];
+  uint64_t grp_full[4];  // per pair of ring items consumed in one step (tiled loads without OWN_P)
   uint64_t s_full[2];
+  uint64_t s_read[2];    // OWN_P: S(j) is in the softmax warps' registers
   uint64_t p_full[2];
-  uint64_t o_done[2];
+  uint64_t o_done[2];    // the last P V is complete; OWN_P: every step's
   uint32_t tmem_base;
   int32_t abort;
 };
+
+static_assert(sizeof(Bars) <= 256, "barrier space");
 
 // workspace header: the number of listed work units sits after the status word
 constexpr size_t kWsItemTotal = 128;
@@ -305,6 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int i = 0; i < C::NGRP; ++i) mbar_init(&bars->grp_full[i], 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->s_full[i], 1);
+      mbar_init(&bars->s_read[i], 4);
       mbar_init(&bars->p_full[i], 128);
       mbar_init(&bars->o_done[i], 1);
     }
@@ -384,8 +399,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           // barrier, armed for both by the first; group 0 (K_0) and group nkv (V_{nkv-1})
           // hold one item
           const int m = (c + 1) >> 1;
-          uint64_t* gb = &bars->grp_full[m % C::NGRP];
-          if (c == 0 || (c & 1)) mbar_arrive_expect_tx(gb, (m == 0 || m == nkv ? 1 : 2) * C::TILE);
+          uint64_t* gb = C::OWN_P ? &bars->kv_full[slot] : &bars->grp_full[m % C::NGRP];
+          if (C::OWN_P)
+            mbar_arrive_expect_tx(gb, C::TILE);
+          else if (c == 0 || (c & 1))
+            mbar_arrive_expect_tx(gb, (m == 0 || m == nkv ? 1 : 2) * C::TILE);
           const CUtensorMap* tm = is_v ? &tm_v : &tm_k;
 #pragma unroll
           for (int kb = 0; kb < C::KB; ++kb)
@@ -393,7 +411,41 @@ __global__ void __launch_bounds__(kThreads, 1)
                              keep_l2);
         }
       }
-    } else if (warp == 1) {
+    } else if (C::OWN_P && (warp == 1 || warp == 2)) {
+    // ---------------------------------------------------- MMA issuers (S; P V)
+      const uint64_t q0d = smem_desc(sbase + C::OFF_Q0, 16, 1024);
+      const uint64_t kv_kmaj = smem_desc(sbase + C::OFF_KV, 16, 1024);
+      const uint64_t kv_mnmaj = smem_desc(sbase + C::OFF_KV, C::BLOCK, 1024);
+      bool ok = warp == 2 || mbar_wait(&bars->q_full, 0);
+      for (int j = 0; ok && j < nkv; ++j) {
+        // ring item of K_j (warp 1) or V_j (warp 2)
+        const int c = warp == 1 ? (j == 0 ? 0 : 2 * j - 1) : (j == nkv - 1 ? 2 * nkv - 1 : 2 * j + 2);
+        const int slot = c % C::NSLOT;
+        ok = mbar_wait(&bars->kv_full[slot], (c / C::NSLOT) & 1);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (!ok || (t == 0 ? j > m0 : !has1)) continue;
+          if (warp == 1) {
+            if (j > 0) ok = mbar_wait(&bars->s_read[t], (j - 1) & 1);
+            tc_fence_after();
+            if (ok && elect_one()) {
+              issue_s<D>(tmem + (t ? C::TM_S1 : C::TM_S0), desc_at(q0d, t * C::TILE), desc_at(kv_kmaj, slot * C::TILE));
+              tc_commit(&bars->s_full[t]);
+            }
+          } else {
+            ok = mbar_wait(&bars->p_full[t], j & 1);
+            tc_fence_after();
+            if (ok && elect_one()) {
+              issue_pv<D>(tmem + (t ? C::TM_O1 : C::TM_O0), tmem + (t ? C::TM_P1 : C::TM_P0),
+                          desc_at(kv_mnmaj, slot * C::TILE), j > 0);
+              tc_commit(&bars->o_done[t]);
+            }
+          }
+          __syncwarp();
+        }
+      }
+      if (!ok) on_timeout(bars, status);
+    } else if (!C::OWN_P && warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     // The whole warp runs the loop and one elected lane issues, so that descriptors and addresses
     // stay in uniform registers; as a one-lane branch each MMA took 75-100 cycles to issue instead of
@@ -495,6 +547,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
       const uint32_t s_col = wg == 0 ? C::TM_S0 : C::TM_S1;
       const uint32_t o_col = wg == 0 ? C::TM_O0 : C::TM_O1;
+      const uint32_t p_col = wg == 0 ? C::TM_P0 : C::TM_P1;
       const uint64_t sc2 = f2pack(scale_log2, scale_log2);
       float m_run = -FLT_MAX, l = 0.f;
       bool ok = true;
@@ -504,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // MMA that reads K_j (the S(j) of both tiles) and V_{j-1} (the P V of both tiles at
       // step j-1), so one thread of that tile's warpgroup frees their slots.  The last V_{n-1}
       // is not handed back: the producer has issued every load by then.
-      const bool releaser = !GATHER && (has1 ? wg == 1 : wg == 0) && quad == 0 && lane == 0;
+      const bool releaser = (!GATHER || C::OWN_P) && (has1 ? wg == 1 : wg == 0) && quad == 0 && lane == 0;
       for (int j = 0; j <= mt; ++j) {
         // S(j) complete also means P(j-1) was consumed and O holds P(j-1) V.  The wait's
         // outcome is the warp's: the TMEM loads and votes below are warp-collective.
@@ -512,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (releaser) {
           // ring items: K_j is 0 for j = 0, else 2j-1; V_{j-1} is 2(j-1)+2 = 2j (j-1 < nkv-1 here)
           mbar_arrive(&bars->kv_empty[(j == 0 ? 0 : 2 * j - 1) % C::NSLOT]);
-          if (j > 0) mbar_arrive(&bars->kv_empty[(2 * j) % C::NSLOT]);
+          if (!C::OWN_P && j > 0) mbar_arrive(&bars->kv_empty[(2 * j) % C::NSLOT]);
         }
         tc_fence_after();
         uint32_t s[128];
@@ -521,6 +574,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_ld_32x32b_x32(trow + s_col + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&s[c * 32]));
         tmem_ld_wait();
         reg_fence<128>(s);
+        if constexpr (C::OWN_P) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->s_read[wg]);
+        }
         if (j == mt) {  // diagonal tile: key c is visible to row r iff c <= r
 #pragma unroll
           for (int c = 0; c < 128; ++c)
@@ -562,9 +620,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         f2unpack(fadd2(acc[0], acc[1]), a0, a1);
         f2unpack(fadd2(acc[2], acc[3]), b0, b1);
         l = l * alpha + ((a0 + a1) + (b0 + b1));
-        // P over the first 64 columns of S (the MMA reads it from there)
-        tmem_st_32x32b_x32(trow + s_col, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
-        tmem_st_32x32b_x32(trow + s_col + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
+        if (C::OWN_P && j > 0) {  // P(j-1) V complete: P's columns are free and O is up to date
+          if (!mbar_wait_warp(&bars->o_done[wg], (j - 1) & 1)) { ok = false; break; }
+          if (releaser) mbar_arrive(&bars->kv_empty[(2 * j) % C::NSLOT]);  // V_{j-1}
+          tc_fence_after();
+        }
+        // P where the MMA reads it from (without OWN_P, the first 64 columns of S)
+        tmem_st_32x32b_x32(trow + p_col, *reinterpret_cast<uint32_t(*)[32]>(&s[0]));
+        tmem_st_32x32b_x32(trow + p_col + 32, *reinterpret_cast<uint32_t(*)[32]>(&s[32]));
         if (j > 0 && __any_sync(0xffffffffu, rescale)) {
           const uint64_t al2 = f2pack(alpha, alpha);
 #pragma unroll
@@ -588,7 +651,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_arrive(&bars->p_full[wg]);
         if (__any_sync(0xffffffffu, aborted(bars))) { ok = false; break; }
       }
-      if (ok) ok = mbar_wait_warp(&bars->o_done[wg], 0);
+      if (ok) ok = mbar_wait_warp(&bars->o_done[wg], C::OWN_P ? mt & 1 : 0);
       if (!ok) {
         on_timeout(bars, status);
       } else {
