@@ -257,7 +257,7 @@ class Path:
                                         self.window, self.keep, self.max_seg, self.max_tok, self.cu_seqlens, None,
                                         self.tok_gather, self.tok_src, self.tok_pos, self.tok_mask,
                                         self.sizes_all[i], self.seg_ws, self.seg_ws_bytes, stream)
-            launches += 5
+            launches += 2 if ci["b1"] - ci["b0"] <= 128 else 3  # plan (and past 128 trajectories write), expand
             assert st == 0, vcs.vcs_status_string(st)
             if evs:
                 evs[1].record(tstream)
@@ -271,13 +271,13 @@ class Path:
                 evs[2].record(tstream)
             st = vcs.vcs_gather(qt, kt, vt, ci["ttok1"] - ci["ttok0"], self.tok_gather, ntok, hq, hkv, d, self.q,
                                 self.k, self.v, self.gstatus, stream)
-            launches += 3
+            launches += 1
             assert st == 0
             if evs:
                 evs[3].record(tstream)
             st = vcs.vcs_attn_fwd(self.q, self.k, self.v, self.cu_seqlens, nseg, ntok, ci["max_seqlen"], hq, hkv,
                                   d, 0.0, self.o, self.lse, self.fwd_ws, self.fwd_ws_bytes, stream)
-            launches += 3  # the work-unit scan and fill, then the attention kernel
+            launches += 3  # the work-unit scan and fill (more than 2,048 units), then the attention kernel
             assert st == 0
             if evs:
                 evs[4].record(tstream)
@@ -288,7 +288,7 @@ class Path:
             st = vcs.vcs_attn_bwd(self.q, self.k, self.v, self.o, self.lse, dout, self.cu_seqlens, nseg, ntok,
                                   ci["max_seqlen"], hq, hkv, d, 0.0, dq, dk, dv, self.bwd_ws, self.bwd_ws_bytes,
                                   stream)
-            launches += 3
+            launches += 3  # D and the zeroed dQ accumulator, the main kernel, dQ's conversion
             assert st == 0
             if evs:
                 evs[5].record(tstream)

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 // at 128 B/clk), TMA writes 64 KB (512), dS^T and the row terms take 512 and the dQ reductions about
 // 990 (measured against a stream of shared loads).  Before, S^T and dP^T were issued together, one
 // pass of the compute warps made P^T and dS^T of both, and dQ left through shared memory by TMA
-// reduce-adds, whose engine also carries the tile loads (64 KB at 25.5 B/clk + 64 KB at 37 B/clk).
+// reduce-adds, whose engine also carries the tile loads (64 KB at 25.5 B/clk + 64 KB at 62 B/clk).
 // vcs_attn_bwd, 40/8/128, four segments of 8,192: 6.18 ms before, 5.31 now (892 -> 1,035 TFLOP/s
 // credited).
 // d = 64: the MMAs need about 1,400 cycles a tile; the compute warps' two passes (about 1,000 and
