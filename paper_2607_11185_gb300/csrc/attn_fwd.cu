@@ -55,8 +55,8 @@
 // d = 64: the MMAs of a step take about 1,020 cycles and the softmax warps bound it, so
 // S_k(j+1) is issued as soon as S_k(j) is in their registers and is complete when they come
 // back for it; before they store P_k(j) they wait for P_k(j-1) V.  One warp issues S and one P V,
-// each waiting for its own ring items.  14/2/64, sixteen segments of 4,096: 0.554 -> 0.523 ms
-// (869 -> 919 TFLOP/s; about 2,100 cycles a step, of which the exponentials of both tiles take
+// each waiting for its own ring items.  14/2/64, sixteen segments of 4,096: 0.554 -> 0.523 ms,
+// 0.513 now (869 -> 937 TFLOP/s; about 2,050 cycles a step, of which the exponentials of both tiles take
 // 1,024 at 32 a clock).
 //
 // Online softmax with a lazy running maximum: the row maximum used for P is
@@ -649,7 +649,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_st_wait();
         tc_fence_before();
         mbar_arrive(&bars->p_full[wg]);
-        if (__any_sync(0xffffffffu, aborted(bars))) { ok = false; break; }
+        // another role's giving up is looked for every eighth step (a shared load and a vote in the
+        // chain that bounds the loop: 14/2/64, sixteen segments of 4,096, 0.523 -> 0.513 ms; a short
+        // batch at 28/4/128 2.09 -> 2.065); the waits are bounded without it
+        if ((j & 7) == 7 && __any_sync(0xffffffffu, aborted(bars))) { ok = false; break; }
       }
       if (ok) ok = mbar_wait_warp(&bars->o_done[wg], C::OWN_P ? mt & 1 : 0);
       if (!ok) {
