@@ -125,7 +125,8 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 //         warp 1: TMEM allocation, MMAs of S^T and dV;  warp 2: MMAs of dP^T, dK and dQ;  warp 3: row terms
 //         (both run warp-uniformly up to an elected lane's issue, which keeps descriptors in uniform
 //         registers: 7.6 -> 6.7 ms on the case above while it was being built)
-//   WG1/2 compute: warpgroup k takes query columns [64k, 64k+64), a thread one key row.  P^T stays
+//   WG1/2 compute: warpgroup k takes query columns [32k, 32k+32) of each half of the tile (so that the
+//         halves' K steps, and with them dK's sum, run in order), a thread one key row.  P^T stays
 //         in fp32 registers between its two passes; its bf16 copy goes to TMEM (the A operand of
 //         dV += P^T dO), dS^T over the dP^T columns the thread has read (A of dK += dS^T Q) and to
 //         shared memory (for dQ)
@@ -176,11 +177,11 @@ struct Bwd {
   static constexpr int TM_DQ = OWN_DQ ? TM_P + 128 : TM_P;
   static constexpr bool OWN_PT = D == 64;
   static constexpr int TM_PT = OWN_PT ? TM_DQ + 64 : TM_S;
-  static constexpr int PT_WG = OWN_PT ? 32 : 64;  // columns from one warpgroup's P^T to the next's
-  // queries [16kk, 16kk+16) of P^T / dS^T: 8 columns of bf16 pairs (each warpgroup's 32 words a row
-  // are at the start of its 64 columns, or alone in P^T's own)
-  __host__ __device__ static constexpr uint32_t pt_col(int kk) { return TM_PT + PT_WG * (kk >> 2) + 8 * (kk & 3); }
-  __host__ __device__ static constexpr uint32_t ds_col(int kk) { return TM_P + 64 * (kk >> 2) + 8 * (kk & 3); }
+  static constexpr int PT_WG = OWN_PT ? 16 : 32;  // columns from one warpgroup's half of P^T to the next's
+  // queries [16kk, 16kk+16) of P^T / dS^T: 8 columns of bf16 pairs (a warpgroup's 16 words of a
+  // half are at the start of its 32 columns, or alone in P^T's own)
+  __host__ __device__ static constexpr uint32_t pt_col(int kk) { return TM_PT + PT_WG * (kk >> 1) + 8 * (kk & 1); }
+  __host__ __device__ static constexpr uint32_t ds_col(int kk) { return TM_P + 32 * (kk >> 1) + 8 * (kk & 1); }
   // Row terms staged by warp 3, or by the compute warps.  d = 64, which the compute warps bound: 1.34
   // ms against 1.29 (14/2/64, sixteen segments of 4,096); d = 128: 0.5% slower by a warp of its own.
   static constexpr bool ROW_WARP = D == 64;
@@ -327,25 +328,33 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
   const int G = hq / hkv;
   const int nsub = (L - n * C::BM + C::BQ - 1) / C::BQ;  // 128-row query tiles at or after this key tile
   const int U = G * nsub;
-  // Tile u covers query rows n*BM + sub_of(u)*BQ ... +BQ-1 of head head_of(u), swept from the
-  // segment end toward the key tile with the G heads of one row block in turn, so that the key
-  // tiles of one (segment, kv head) running together meet the same Q/dO/dQ lines in L2.
+  // Tile u covers query rows n*BM + sub*BQ ... +BQ-1 of one head.  d = 128: swept from the segment
+  // end toward the key tile with the G heads of one row block in turn, so that the key tiles of one
+  // (segment, kv head) running together meet the same Q/dO/dQ lines in L2.  d = 64: head by head
+  // from the key tile to the segment end, which is the order dK and dV are summed in, and the key
+  // tiles that run together are on different rows of dQ.
   struct Walk {  // tile u's row block and head, stepped without divisions
-    int sub, head, g0, G;
+    int sub, head, first, count;  // first head and heads (d = 128); row blocks and last head + 1 (d = 64)
     __device__ __forceinline__ void next() {
-      if (++head == g0 + G) {
-        head = g0;
+      if constexpr (D == 64) {
+        if (++sub == first) {
+          sub = 0;
+          ++head;
+        }
+      } else if (++head == first + count) {
+        head = first;
         --sub;
       }
     }
+    __device__ __forceinline__ bool live() const { return D == 64 ? head < count : sub >= 0; }
   };
-  const Walk walk0{nsub - 1, g * G, g * G, G};
+  const Walk walk0 = D == 64 ? Walk{0, g * G, nsub, g * G + G} : Walk{nsub - 1, g * G, g * G, G};
   // lse and D of query i of w's tile, as loaded: scaled only where they are staged
   auto row_terms = [&](const Walk& w, int i, bool mine, float& l, float& dd) {
     l = __int_as_float(0x7f800000);  // +inf: query outside the segment -> P = 0
     dd = 0.f;
     const int q = n * C::BM + w.sub * C::BQ + i;
-    if (w.sub >= 0 && mine && q < L) {
+    if (w.live() && mine && q < L) {
       const size_t j = (size_t)w.head * num_tokens + start + q;
       l = __ldg(&lse[j]);
       dd = __ldg(&dvec[j]);
@@ -558,7 +567,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
             if (elect_one()) {
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
-                const int kk = 4 * (j >> 1) + 2 * hf + (j & 1);
+                const int kk = 4 * hf + j;
                 tc_mma_ts(tmem + C::TM_DK, tmem + C::ds_col(kk), desc_at(qmn, kk * 2048), C::IDESC_KV,
                           (u > 0 || hf > 0 || j > 0) ? 1u : 0u);
               }
@@ -603,8 +612,8 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       for (int u = 0; u < U; ++u) {
         if (u >= 2 && !mbar_wait_warp(&bars->rt_free[u & 1], ((u >> 1) - 1) & 1)) { ok = false; break; }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {  // warpgroup i/2's 64 queries: nl, then nd
-          float* r = rows + (u & 1) * 256 + (i >> 1) * 128 + (i & 1) * 32 + lane;
+        for (int i = 0; i < 4; ++i) {  // half i/2 of warpgroup i%2's 64 queries: nl, then nd
+          float* r = rows + (u & 1) * 256 + (i & 1) * 128 + (i >> 1) * 32 + lane;
           r[0] = -l[i] * 1.4426950408889634f;
           r[64] = -dd[i] * scale;
         }
@@ -620,13 +629,14 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
   } else if (warp < 12) {
     // ------------------------------------------------------------ compute
     setmaxnreg_inc<C::REG_COMPUTE>();
-    const int k = (warp - 4) >> 2;   // query columns [64k, 64k+64) of the tile
+    // query columns [32k, 32k+32) of each 64-column half of the tile: columns 0..31 and 32..63 below
+    const int k = (warp - 4) >> 2;
     const int quad = warp & 3;
     const int r = quad * 32 + lane;  // TMEM lane: key row
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
     // row terms of the warpgroup's 64 queries: nl = -lse*log2e, then nd = -D*scale; two buffers
     const uint32_t rt_u32 = smem_u32(smem + C::OFF_ROW) + k * 512;
-    const uint32_t ds_row = sbase + C::OFF_DS + k * C::BLOCK + r * 128;
+    const uint32_t ds_row = sbase + C::OFF_DS + r * 128;
     const uint64_t sl2 = f2pack(scale_log2, scale_log2), sc2 = f2pack(scale, scale);
     Walk wc = walk0;  // of the tile computed
     bool ok = true;
@@ -636,7 +646,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     Walk wr = walk0;
     float l0, d0, l1, d1;
     auto next_terms = [&](float& l, float& dd) {
-      row_terms(wr, 64 * k + tw, tw < 64, l, dd);
+      row_terms(wr, 64 * (tw >> 5) + 32 * k + (tw & 31), tw < 64, l, dd);
       wr.next();
     };
     if constexpr (!C::ROW_WARP) {
@@ -645,8 +655,8 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     }
     for (int u = 0; u < U; ++u) {
       // the query rows are the key tile's own: mask keys after queries (column c of the
-      // warpgroup is hidden from key row r when c < dlim)
-      const int dlim = wc.sub == 0 ? r - 64 * k : 0;
+      // warpgroup's half hf is hidden from key row r when c < dlim - 64 hf)
+      const int dlim = wc.sub == 0 ? r - 32 * k : 0;
       wc.next();
       const uint32_t rt = rt_u32 + (u & 1) * 1024;
       if constexpr (!C::ROW_WARP) {
@@ -678,8 +688,8 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       if (C::ROW_WARP) first_terms(rt);
       // P^T = 2^(S^T * scale*log2e - lse*log2e), fp32 in p, bf16 over the S^T columns just read
       uint32_t p[2][32];
-      tmem_ld_cols<32>(trow + C::TM_S + 64 * k, p[0]);
-      tmem_ld_cols<32>(trow + C::TM_S + 64 * k + 32, p[1]);
+      tmem_ld_cols<32>(trow + C::TM_S + 32 * k, p[0]);
+      tmem_ld_cols<32>(trow + C::TM_S + 32 * k + 64, p[1]);
       tmem_ld_wait();
       reg_fence<32>(p[0]);
       reg_fence<32>(p[1]);
@@ -706,16 +716,17 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           x[x0 + c] = __float_as_uint(ex2(a));
           x[x0 + c + 1] = __float_as_uint(ex2(b));
         }
-        if (dlim > 16 * ch) {
+        const int hide = dlim - 64 * (ch >> 1) - x0;
+        if (hide > 0) {
 #pragma unroll
           for (int c = 0; c < 16; ++c)
-            if (16 * ch + c < dlim) x[x0 + c] = 0u;
+            if (c < hide) x[x0 + c] = 0u;
         }
         uint32_t pk[8];
 #pragma unroll
         for (int c2 = 0; c2 < 8; ++c2)
           pk[c2] = pack_bf16(__uint_as_float(x[x0 + 2 * c2]), __uint_as_float(x[x0 + 2 * c2 + 1]));
-        tmem_st_32x32b_x8(trow + C::TM_PT + C::PT_WG * k + 8 * ch, pk);
+        tmem_st_32x32b_x8(trow + C::TM_PT + C::PT_WG * (k + (ch & 2)) + 8 * (ch & 1), pk);
       }
       tmem_st_wait();
       tc_fence_before();
@@ -729,14 +740,14 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       tc_fence_after();
       // dS^T = P^T (dP^T - D) * scale, 16 columns at a time, the next ones' loads in flight
       uint32_t dp[2][16];
-      tmem_ld_cols<16>(trow + C::TM_P + 64 * k, dp[0]);
+      tmem_ld_cols<16>(trow + C::TM_P + 32 * k, dp[0]);
       tmem_ld_wait();
       reg_fence<16>(dp[0]);
 #pragma unroll
       for (int ch = 0; ch < 4; ++ch) {
         const int cur = ch & 1;
         if (ch < 3) {
-          tmem_ld_cols<16>(trow + C::TM_P + 64 * k + 16 * (ch + 1), dp[cur ^ 1]);
+          tmem_ld_cols<16>(trow + C::TM_P + 32 * k + 64 * ((ch + 1) >> 1) + 16 * ((ch + 1) & 1), dp[cur ^ 1]);
 #pragma unroll
           for (int j = 0; j < 4; ++j) rq[cur ^ 1][j] = ld_shared_v4(rt + 256 + 64 * (ch + 1) + 16 * j);
         }
@@ -754,9 +765,9 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-          st_shared_v4(ds_row + (u % C::NDS) * 2 * C::BLOCK + (uint32_t)(((2 * ch + j) ^ (r & 7)) << 4),
+          st_shared_v4(ds_row + ((u % C::NDS) * 2 + (ch >> 1)) * C::BLOCK + (uint32_t)(((4 * k + 2 * (ch & 1) + j) ^ (r & 7)) << 4),
                        wd[4 * j], wd[4 * j + 1], wd[4 * j + 2], wd[4 * j + 3]);
-        tmem_st_32x32b_x8(trow + C::TM_P + 64 * k + 8 * ch, wd);
+        tmem_st_32x32b_x8(trow + C::TM_P + 32 * k + 64 * (ch >> 1) + 8 * (ch & 1), wd);
         if (ch & 1) {
           // dQ, the only reader of dS^T in shared memory, is issued after both halves' barriers, so
           // the second half's fence serves both (each costs the warp a drain of its stores: one

@@ -218,3 +218,40 @@ def test_query_tile_counts_around_the_rings(hq, hkv, d):
     for name, got, ref in (("dq", dq, rq), ("dk", dk, rk), ("dv", dv, rv)):
         e = rel_err(got.float().cpu().numpy(), ref)
         assert e <= REL, (name, e)
+
+
+def test_dk_dv_summed_in_query_order_d64():
+    """At d = 64 dK and dV are fp32 sums over the group's heads in turn, each from the key tile's own
+    rows to the segment end, 16 query rows a term.  Every dim gets a 1, a 2^30 and a -2^30 in three of
+    the terms, whose sum is 1 or 0 by their order, so the result is that order's, exactly."""
+    d, G, L, big = 64, 2, 384 + 40, float(2 ** 30)
+    rng = np.random.default_rng(3)
+    groups = (L + 15) // 16
+    order = [(h, c) for h in range(G) for c in range(groups)]
+
+    def column():
+        terms = np.zeros(len(order), np.float32)
+        at = rng.choice(len(order), 3, replace=False)
+        terms[at] = rng.permutation([1.0, big, -big])
+        total = np.float32(0)
+        for t in terms:
+            total = np.float32(total + t)
+        return terms, total
+
+    # keys 0 and 1 share every later row (P = 1/2 each), with opposite values: O = 0, dS = +-1
+    q = torch.zeros(L, G, d)
+    do = torch.zeros(L, G, d)
+    k = torch.zeros(L, 1, d)
+    v = torch.zeros(L, 1, d)
+    q[:, :, 0], do[:, :, 0], k[:2, 0, 0], k[2:, 0, 0] = 16, 16, 16, -16
+    v[0, 0, 0], v[1, 0, 0] = 1, -1
+    want = np.zeros((2, d), np.float32)  # dK_0 and dV_0
+    for b in range(1, d):
+        for which, (x, unit) in enumerate(((q, 1.0), (do, 2.0))):
+            terms, want[which, b] = column()
+            for (h, c), t in zip(order, terms):
+                x[min(16 * c + 1 + int(rng.integers(0, 15)), L - 1), h, b] = unit * float(t)
+    _, _, _, dk, dv = run(*(x.bfloat16().cuda() for x in (q, k, v, do)), [0, L])
+    assert 8 < want[0].sum() < d - 8 and 8 < want[1].sum() < d - 8  # both outcomes occur
+    assert np.array_equal(dk[0, 0, 1:].float().cpu().numpy(), want[0, 1:])
+    assert np.array_equal(dv[0, 0, 1:].float().cpu().numpy(), want[1, 1:])
