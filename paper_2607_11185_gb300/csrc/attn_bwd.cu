@@ -491,35 +491,31 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           tc_mma_ss(tm, desc_at(a, o), desc_at(b, o), C::IDESC_S, kk > 0);
         }
       };
+      // A wait can run out, and another role give up, between two lanes' reads, so no lane's answer
+      // decides where the warp goes: every lane runs every tile, one that has given up waits no more, and
+      // the elected lane issues as long as its own waits were met.
       bool ok = mbar_wait(&bars->kv_full, 0);
       if (warp == 1) {
         // S^T and dV.  d = 128: S^T(u+1) overwrites P^T(u), which dV(u), issued before, reads first.
         // d = 64: P^T has columns of its own, so S^T(u+1) is issued as soon as S^T(u) is read; its
         // barrier is then completed by dV(u), which also frees P^T's columns.
-        auto issue_s = [&](int u) -> bool {
-          if (!mbar_wait(&bars->q_full[u % C::NST], (u / C::NST) & 1)) return false;
-          if (C::OWN_PT && u > 0 && !mbar_wait(&bars->s_read, (u - 1) & 1)) return false;
+        auto issue_s = [&](int u) {
+          ok = ok && mbar_wait(&bars->q_full[u % C::NST], (u / C::NST) & 1);
+          if (C::OWN_PT && u > 0) ok = ok && mbar_wait(&bars->s_read, (u - 1) & 1);
           tc_fence_after();
-          if (elect_one()) {
+          if (elect_one() && ok) {
             issue_kmaj(tmem + C::TM_S, k_kmaj, desc_at(qd_kmaj, C::q_off(u)));
             if (!C::OWN_PT || u == 0) tc_commit(&bars->s_full);
           }
           __syncwarp();
-          return true;
         };
-        ok = ok && issue_s(0);
-        for (int u = 0; ok && u < U; ++u) {
-          if (C::OWN_PT && u + 1 < U && !issue_s(u + 1)) {
-            ok = false;
-            break;
-          }
-          if (!mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1) || !mbar_wait(&bars->p_full, u & 1) ||
-              aborted_now()) {
-            ok = false;
-            break;
-          }
+        issue_s(0);
+        for (int u = 0; u < U; ++u) {
+          if (C::OWN_PT && u + 1 < U) issue_s(u + 1);
+          ok = ok && mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1) && mbar_wait(&bars->p_full, u & 1) &&
+               !aborted_now();
           tc_fence_after();
-          if (elect_one()) {
+          if (elect_one() && ok) {
             const uint64_t dmn = desc_at(qd_mnmaj, C::do_off(u));
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)
@@ -529,7 +525,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
             if (C::OWN_PT && u + 1 < U) tc_commit(&bars->s_full);
           }
           __syncwarp();
-          if (!C::OWN_PT && u + 1 < U) ok = issue_s(u + 1);
+          if (!C::OWN_PT && u + 1 < U) issue_s(u + 1);
         }
       } else {
         // dP^T, dK and dQ.  d = 128: dP^T(u) goes where dQ(u-1) was, dQ(u) where dS^T(u) was, which
@@ -538,33 +534,28 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         // next); dS^T in shared memory then takes two buffers.
         const uint64_t v_kmaj = desc_at(k_kmaj, C::OFF_V);
         const uint64_t ds_mnmaj = desc_at(k_mnmaj, C::OFF_DS);
-        auto issue_dp = [&](int u) -> bool {
-          if (!mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1) ||
-              (!C::OWN_DQ && u > 0 && !mbar_wait(&bars->dq_free, (u - 1) & 1)) || aborted_now())
-            return false;
+        auto issue_dp = [&](int u) {
+          ok = ok && mbar_wait(&bars->do_full[u % C::NST], (u / C::NST) & 1);
+          if (!C::OWN_DQ && u > 0) ok = ok && mbar_wait(&bars->dq_free, (u - 1) & 1);
+          ok = ok && !aborted_now();
           tc_fence_after();
-          if (elect_one()) {
+          if (elect_one() && ok) {
             issue_kmaj(tmem + C::TM_P, v_kmaj, desc_at(qd_kmaj, C::do_off(u)));
             tc_commit(&bars->dp_full);
             mbar_arrive(&bars->p_full);
             tc_commit(&bars->do_done[u % C::NST]);
           }
           __syncwarp();
-          return true;
         };
-        if (C::OWN_DQ) ok = ok && issue_dp(0);
-        for (int u = 0; ok && u < U; ++u) {
-          if (!C::OWN_DQ && !issue_dp(u)) {
-            ok = false;
-            break;
-          }
+        if (C::OWN_DQ) issue_dp(0);
+        for (int u = 0; u < U; ++u) {
+          if (!C::OWN_DQ) issue_dp(u);
           const uint64_t qmn = desc_at(qd_mnmaj, C::q_off(u));
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
-            if (ok && !mbar_wait(&bars->ds_full[hf], u & 1)) ok = false;
-            if (!ok) break;
+            ok = ok && mbar_wait(&bars->ds_full[hf], u & 1);
             tc_fence_after();
-            if (elect_one()) {
+            if (elect_one() && ok) {
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
                 const int kk = 4 * hf + j;
@@ -575,12 +566,11 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
             __syncwarp();
           }
           if (C::OWN_DQ) {
-            if (ok && u + 1 < U) ok = issue_dp(u + 1);
-            if (ok && u > 0) ok = mbar_wait(&bars->dq_free, (u - 1) & 1);
+            if (u + 1 < U) issue_dp(u + 1);
+            if (u > 0) ok = ok && mbar_wait(&bars->dq_free, (u - 1) & 1);
             tc_fence_after();
           }
-          if (!ok) break;
-          if (elect_one()) {
+          if (elect_one() && ok) {
             const uint64_t ds = desc_at(ds_mnmaj, (u % C::NDS) * 2 * C::BLOCK);
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk)

@@ -416,26 +416,29 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t q0d = smem_desc(sbase + C::OFF_Q0, 16, 1024);
       const uint64_t kv_kmaj = smem_desc(sbase + C::OFF_KV, 16, 1024);
       const uint64_t kv_mnmaj = smem_desc(sbase + C::OFF_KV, C::BLOCK, 1024);
+      // A wait can run out between two lanes' reads, so no lane's answer decides where the warp goes:
+      // every lane runs every step, one that has given up waits no more, and the elected lane issues as
+      // long as its own waits were met.
       bool ok = warp == 2 || mbar_wait(&bars->q_full, 0);
-      for (int j = 0; ok && j < nkv; ++j) {
+      for (int j = 0; j < nkv; ++j) {
         // ring item of K_j (warp 1) or V_j (warp 2)
         const int c = warp == 1 ? (j == 0 ? 0 : 2 * j - 1) : (j == nkv - 1 ? 2 * nkv - 1 : 2 * j + 2);
         const int slot = c % C::NSLOT;
-        ok = mbar_wait(&bars->kv_full[slot], (c / C::NSLOT) & 1);
+        ok = ok && mbar_wait(&bars->kv_full[slot], (c / C::NSLOT) & 1);
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-          if (!ok || (t == 0 ? j > m0 : !has1)) continue;
+          if (t == 0 ? j > m0 : !has1) continue;
           if (warp == 1) {
-            if (j > 0) ok = mbar_wait(&bars->s_read[t], (j - 1) & 1);
+            if (j > 0) ok = ok && mbar_wait(&bars->s_read[t], (j - 1) & 1);
             tc_fence_after();
-            if (ok && elect_one()) {
+            if (elect_one() && ok) {
               issue_s<D>(tmem + (t ? C::TM_S1 : C::TM_S0), desc_at(q0d, t * C::TILE), desc_at(kv_kmaj, slot * C::TILE));
               tc_commit(&bars->s_full[t]);
             }
           } else {
-            ok = mbar_wait(&bars->p_full[t], j & 1);
+            ok = ok && mbar_wait(&bars->p_full[t], j & 1);
             tc_fence_after();
-            if (ok && elect_one()) {
+            if (elect_one() && ok) {
               issue_pv<D>(tmem + (t ? C::TM_O1 : C::TM_O0), tmem + (t ? C::TM_P1 : C::TM_P0),
                           desc_at(kv_mnmaj, slot * C::TILE), j > 0);
               tc_commit(&bars->o_done[t]);
@@ -450,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The whole warp runs the loop and one elected lane issues, so that descriptors and addresses
     // stay in uniform registers; as a one-lane branch each MMA took 75-100 cycles to issue instead of
     // the 64 it executes in (four segments of 8,192 at 40/8/128: 1.774 -> 1.674 ms, sixteen of 4,096
-    // at 14/2/64: 0.618 -> 0.562).
+    // at 14/2/64: 0.618 -> 0.562).  As above, no lane's answer decides where the warp goes.
       bool ok = mbar_wait(&bars->q_full, 0);
       // descriptors built once; the issue loops only add compile-time offsets
       const uint64_t q0d = smem_desc(sbase + C::OFF_Q0, 16, 1024), q1d = desc_at(q0d, C::TILE);
@@ -463,20 +466,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto v_off = [&](int j) { return (uint32_t)((v_item(j) % C::NSLOT) * C::TILE); };
       // tiled loads: group m holds K_m and V_{m-1} (group 0 only K_0, group nkv only
       // V_{nkv-1}); gathered loads: one barrier per ring item
-      auto acquire_group = [&](int m) -> bool {
+      auto acquire_group = [&](int m) {
         if constexpr (GATHER) {
-          if (m < nkv && !mbar_wait(&bars->kv_full[k_item(m) % C::NSLOT], (k_item(m) / C::NSLOT) & 1)) return false;
-          if (m > 0 && !mbar_wait(&bars->kv_full[v_item(m - 1) % C::NSLOT], (v_item(m - 1) / C::NSLOT) & 1))
-            return false;
+          if (m < nkv) ok = ok && mbar_wait(&bars->kv_full[k_item(m) % C::NSLOT], (k_item(m) / C::NSLOT) & 1);
+          if (m > 0) ok = ok && mbar_wait(&bars->kv_full[v_item(m - 1) % C::NSLOT], (v_item(m - 1) / C::NSLOT) & 1);
         } else {
-          if (!mbar_wait(&bars->grp_full[m % C::NGRP], (m / C::NGRP) & 1)) return false;
+          ok = ok && mbar_wait(&bars->grp_full[m % C::NGRP], (m / C::NGRP) & 1);
         }
         tc_fence_after();
-        return true;
       };
       uint32_t kaddr = k_off(0), vaddr = 0;  // slot byte offsets of K_{j+1} and V_j
-      if (ok) ok = acquire_group(0);
-      if (ok && elect_one()) {
+      acquire_group(0);
+      if (elect_one() && ok) {
         issue_s<D>(tmem + C::TM_S0, q0d, desc_at(kv_kmaj, kaddr));
         tc_commit(&bars->s_full[0]);
         if (has1) {
@@ -490,16 +491,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       // step (a barrier wait stalls the issuing thread for hundreds of cycles while the pipe
       // streams from shared memory, so the fewer the better), a step after the producer asked
       // for it
-      for (int j = 0; ok && j < nkv; ++j) {
+      for (int j = 0; j < nkv; ++j) {
         const bool next = j + 1 < nkv;
-        if (!acquire_group(j + 1)) { ok = false; break; }
+        acquire_group(j + 1);
         vaddr = v_off(j);
         if (next) kaddr = k_off(j + 1);
         // tile 0: O0 += P0(j) V_j, then S0(j+1)
         if (j <= m0) {
-          if (!mbar_wait(&bars->p_full[0], j & 1)) { ok = false; break; }
+          ok = ok && mbar_wait(&bars->p_full[0], j & 1);
           tc_fence_after();
-          if (elect_one()) {
+          if (elect_one() && ok) {
             issue_pv<D>(tmem + C::TM_O0, tmem + C::TM_S0, desc_at(kv_mnmaj, vaddr), j > 0);
             if (next && j + 1 <= m0) {
               issue_s<D>(tmem + C::TM_S0, q0d, desc_at(kv_kmaj, kaddr));
@@ -512,9 +513,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // tile 1
         if (has1) {
-          if (!mbar_wait(&bars->p_full[1], j & 1)) { ok = false; break; }
+          ok = ok && mbar_wait(&bars->p_full[1], j & 1);
           tc_fence_after();
-          if (elect_one()) {
+          if (elect_one() && ok) {
             issue_pv<D>(tmem + C::TM_O1, tmem + C::TM_S1, desc_at(kv_mnmaj, vaddr), j > 0);
             if (next) {
               issue_s<D>(tmem + C::TM_S1, q1d, desc_at(kv_kmaj, kaddr));
@@ -527,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if constexpr (GATHER) {
           // the gathering producer needs its slots back as soon as the MMAs are done with them
-          if (elect_one()) {
+          if (elect_one() && ok) {
             if (next) tc_commit(&bars->kv_empty[k_item(j + 1) % C::NSLOT]);
             tc_commit(&bars->kv_empty[v_item(j) % C::NSLOT]);
           }
