@@ -271,13 +271,19 @@ def _host_words(n: int, dtype) -> torch.Tensor:
     return t
 
 
+def _torch_stream(stream) -> torch.cuda.Stream:
+    """`stream` as the raw calls take it (None, a stream object or a handle) as a torch stream."""
+    if stream is None:
+        return torch.cuda.current_stream()
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    handle = _stream(stream)  # torch makes a new stream of the handle 0, the default stream's
+    return torch.cuda.ExternalStream(handle) if handle else torch.cuda.default_stream()
+
+
 def _wait(stream):
     """Blocks until the work issued so far on the call's stream is done."""
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    elif isinstance(stream, int):
-        stream = torch.cuda.ExternalStream(stream)
-    stream.synchronize()
+    _torch_stream(stream).synchronize()
 
 
 def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stream=None):
