@@ -12,6 +12,8 @@ non-zero status.
 from __future__ import annotations
 
 import ctypes
+import functools
+import inspect
 import math
 import os
 from typing import Optional
@@ -272,38 +274,71 @@ def _host_words(n: int, dtype) -> torch.Tensor:
 
 
 def _torch_stream(stream) -> torch.cuda.Stream:
-    """`stream` as the raw calls take it (None, a stream object or a handle) as a torch stream."""
-    if stream is None:
-        return torch.cuda.current_stream()
+    """`stream` as the raw calls take it (a stream object or a handle) as a torch stream."""
     if isinstance(stream, torch.cuda.Stream):
         return stream
     handle = _stream(stream)  # torch makes a new stream of the handle 0, the default stream's
     return torch.cuda.ExternalStream(handle) if handle else torch.cuda.default_stream()
 
 
-def _wait(stream):
-    """Blocks until the work issued so far on the call's stream is done."""
-    _torch_stream(stream).synchronize()
+def _wait():
+    """Blocks until the work issued so far on the call's stream, the current one, is done."""
+    torch.cuda.current_stream().synchronize()
 
 
+def _tensors(x):
+    if isinstance(x, torch.Tensor):
+        yield x
+    elif isinstance(x, (tuple, dict)):
+        for y in x.values() if isinstance(x, dict) else x:
+            yield from _tensors(y)
+
+
+def _on_stream(fn):
+    """Runs a convenience with its `stream` as the current one, so that the workspace and the outputs come
+    from that stream's memory pool and the status words are read in that stream's order.  The outputs are
+    marked as used by the caller's current stream, where the caller goes on with them."""
+    at = list(inspect.signature(fn).parameters).index("stream")
+
+    @functools.wraps(fn)
+    def call(*args, **kwargs):
+        given = args[at] if len(args) > at else kwargs.pop("stream", None)
+        if given is None:
+            return fn(*args, **kwargs)
+        if len(args) > at:
+            args = (*args[:at], None, *args[at + 1:])
+        caller, stream = torch.cuda.current_stream(), _torch_stream(given)
+        if stream == caller:
+            return fn(*args, **kwargs)
+        with torch.cuda.stream(stream):
+            out = fn(*args, **kwargs)
+        for t in _tensors(out):
+            t.record_stream(caller)
+        return out
+
+    return call
+
+
+@_on_stream
 def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stream=None):
     """Segment count, token count and longest segment (synchronises once)."""
     dev = cu_steps.device
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
     nb = vcs_segments_workspace_size(num_traj, num_steps)
-    return _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, _ws(nb, dev), nb, stream)
+    return _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, _ws(nb, dev), nb)
 
 
-def _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb, stream):
+def _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb):
     sizes = _host_words(3, torch.int64)   # 24 bytes = vcs_sizes
-    _check(vcs_plan_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, nb,
-                             stream), "vcs_plan_segments")
-    _wait(stream)
+    _check(vcs_plan_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, nb),
+           "vcs_plan_segments")
+    _wait()
     ns, nt, tail = sizes.tolist()
     _check(tail >> 32, "vcs_plan_segments (device)")
     return ns, nt, tail & 0xFFFFFFFF
 
 
+@_on_stream
 def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, with_mask: bool = True,
                    stream=None):
     """Plan + build: returns a dict of device tensors and the sizes."""
@@ -311,7 +346,7 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
     nb = vcs_segments_workspace_size(num_traj, num_steps)
     ws = _ws(nb, dev)
-    ns, nt, mx = _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb, stream)
+    ns, nt, mx = _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb)
     sizes = _host_words(3, torch.int64)
     out = dict(cu_seqlens=torch.empty(ns + 1, dtype=torch.int32, device=dev),
                seg_traj=torch.empty(ns, dtype=torch.int32, device=dev),
@@ -321,13 +356,14 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
                tok_loss_mask=torch.empty(nt, dtype=torch.uint8, device=dev) if with_mask else None)
     _check(vcs_build_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ns, nt,
                               out["cu_seqlens"], out["seg_traj"], out["tok_gather"], out["tok_src_step"],
-                              out["tok_pos"], out["tok_loss_mask"], sizes, ws, nb, stream), "vcs_build_segments")
-    _wait(stream)
+                              out["tok_pos"], out["tok_loss_mask"], sizes, ws, nb), "vcs_build_segments")
+    _wait()
     _check(sizes.tolist()[2] >> 32, "vcs_build_segments (device)")
     out.update(num_segments=ns, num_tokens=nt, max_seqlen=mx)
     return out
 
 
+@_on_stream
 def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
     nt = tok_gather.numel()
     _, hq, d = q_traj.shape
@@ -337,13 +373,14 @@ def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
     k = torch.empty((nt, hkv, d), dtype=k_traj.dtype, device=dev)
     v = torch.empty((nt, hkv, d), dtype=v_traj.dtype, device=dev)
     status = _host_words(1, torch.int32)
-    _check(vcs_gather(q_traj, k_traj, v_traj, q_traj.shape[0], tok_gather, nt, hq, hkv, d, q, k, v, status,
-                      stream), "vcs_gather")
-    _wait(stream)
+    _check(vcs_gather(q_traj, k_traj, v_traj, q_traj.shape[0], tok_gather, nt, hq, hkv, d, q, k, v, status),
+           "vcs_gather")
+    _wait()
     _check(status.tolist()[0], "vcs_gather (device)")
     return q, k, v
 
 
+@_on_stream
 def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, stream=None, check=True):
     nt, hq, d = q.shape
     hkv = k.shape[1]
@@ -352,13 +389,14 @@ def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, s
     lse = torch.empty((hq, nt), dtype=torch.float32, device=q.device)
     nb = vcs_attn_fwd_workspace_size(ns, nt, max_seqlen, hq, hkv, d)
     ws = _ws(nb, q.device)
-    _check(vcs_attn_fwd(q, k, v, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, o, lse, ws, nb,
-                        stream), "vcs_attn_fwd")
+    _check(vcs_attn_fwd(q, k, v, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, o, lse, ws, nb),
+           "vcs_attn_fwd")
     if check:
         _check(int(ws[0].item()), "vcs_attn_fwd (device)")
     return o, lse
 
 
+@_on_stream
 def attn_bwd(q, k, v, o, lse, dout, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, stream=None,
              check=True):
     nt, hq, d = q.shape
@@ -368,24 +406,26 @@ def attn_bwd(q, k, v, o, lse, dout, cu_seqlens, max_seqlen: int, softmax_scale: 
     nb = vcs_attn_bwd_workspace_size(ns, nt, max_seqlen, hq, hkv, d)
     ws = _ws(nb, q.device)
     _check(vcs_attn_bwd(q, k, v, o, lse, dout, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, dq, dk,
-                        dv, ws, nb, stream), "vcs_attn_bwd")
+                        dv, ws, nb), "vcs_attn_bwd")
     if check:
         _check(int(ws[0].item()), "vcs_attn_bwd (device)")
     return dq, dk, dv
 
 
+@_on_stream
 def shared_prefix(cu_seqlens, seg_traj, tok_gather, stream=None):
     """Per segment, its common prefix length with the previous segment of its trajectory."""
     ns = cu_seqlens.numel() - 1
     out = torch.empty(max(ns, 0), dtype=torch.int32, device=cu_seqlens.device)
     status = _host_words(1, torch.int32)
-    _check(vcs_shared_prefix(cu_seqlens, seg_traj, tok_gather, ns, tok_gather.numel(), out, status, stream),
+    _check(vcs_shared_prefix(cu_seqlens, seg_traj, tok_gather, ns, tok_gather.numel(), out, status),
            "vcs_shared_prefix")
-    _wait(stream)
+    _wait()
     _check(status.tolist()[0], "vcs_shared_prefix (device)")
     return out
 
 
+@_on_stream
 def attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, max_seqlen: int, softmax_scale: float = 0.0, stream=None,
                    check=True):
     """vcs_attn_fwd's o and lse, computing each shared prefix row once per trajectory."""
@@ -397,12 +437,13 @@ def attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, max_seqlen: int, softmax_sca
     nb = vcs_attn_fwd_workspace_size(ns, nt, max_seqlen, hq, hkv, d)
     ws = _ws(nb, q.device)
     _check(vcs_attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, ns, nt, max_seqlen, hq, hkv, d, softmax_scale, o, lse,
-                              ws, nb, stream), "vcs_attn_fwd_reuse")
+                              ws, nb), "vcs_attn_fwd_reuse")
     if check:
         _check(int(ws[0].item()), "vcs_attn_fwd_reuse (device)")
     return o, lse
 
 
+@_on_stream
 def attn_fwd_gathered(q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0,
                       stream=None, check=True):
     """Attention forward over the segments, reading trajectory-layout q/k/v through tok_gather;
@@ -416,12 +457,13 @@ def attn_fwd_gathered(q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen
     nb = vcs_attn_fwd_workspace_size(ns, nt, max_seqlen, hq, hkv, d)
     ws = _ws(nb, q_traj.device)
     _check(vcs_attn_fwd_gathered(q_traj, k_traj, v_traj, tt, tok_gather, cu_seqlens, ns, nt, max_seqlen, hq, hkv, d,
-                                 softmax_scale, o, lse, ws, nb, stream), "vcs_attn_fwd_gathered")
+                                 softmax_scale, o, lse, ws, nb), "vcs_attn_fwd_gathered")
     if check:
         _check(int(ws[0].item()), "vcs_attn_fwd_gathered (device)")
     return o, lse
 
 
+@_on_stream
 def attn_bwd_gathered(q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqlens, max_seqlen: int,
                       softmax_scale: float = 0.0, stream=None, check=True):
     """Attention backward over the segments with trajectory-layout q/k/v read through tok_gather;
@@ -434,13 +476,14 @@ def attn_bwd_gathered(q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqle
     nb = vcs_attn_bwd_gathered_workspace_size(ns, nt, max_seqlen, tt, hq, hkv, d)
     ws = _ws(nb, q_traj.device)
     _check(vcs_attn_bwd_gathered(q_traj, k_traj, v_traj, tt, tok_gather, o, lse, dout, cu_seqlens, ns, nt,
-                                 max_seqlen, hq, hkv, d, softmax_scale, dq, dk, dv, ws, nb, stream),
+                                 max_seqlen, hq, hkv, d, softmax_scale, dq, dk, dv, ws, nb),
            "vcs_attn_bwd_gathered")
     if check:
         _check(int(ws[0].item()), "vcs_attn_bwd_gathered (device)")
     return dq, dk, dv
 
 
+@_on_stream
 def grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv, eps_low: float = 0.2,
               eps_high: float = 0.28, clip_cap: float = 3.0, kl_coef: float = 1e-4, with_grad: bool = True,
               stream=None, check=True):
@@ -452,13 +495,14 @@ def grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv
     nb = vcs_grpo_loss_workspace_size(nt)
     ws = _ws(nb, dev)
     _check(vcs_grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, seg_traj.numel(), nt, adv,
-                         adv.numel(), eps_low, eps_high, clip_cap, kl_coef, loss, dlogp, ws, nb, stream),
+                         adv.numel(), eps_low, eps_high, clip_cap, kl_coef, loss, dlogp, ws, nb),
            "vcs_grpo_loss")
     if check:
         _check(int(ws[0].item()), "vcs_grpo_loss (device)")
     return loss, dlogp
 
 
+@_on_stream
 def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     """(ids int32, logp fp32) of every segment token (Algorithm 1's stream fields)."""
     nt = tok_gather.numel()
@@ -466,13 +510,14 @@ def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     ids = torch.empty(nt, dtype=torch.int32, device=dev)
     logp = torch.empty(nt, dtype=torch.float32, device=dev)
     status = _host_words(1, torch.int32)
-    _check(vcs_stream_fields(traj_ids, traj_logp, traj_ids.numel(), tok_gather, tok_loss_mask, nt, ids, logp, status,
-                             stream), "vcs_stream_fields")
-    _wait(stream)
+    _check(vcs_stream_fields(traj_ids, traj_logp, traj_ids.numel(), tok_gather, tok_loss_mask, nt, ids, logp, status),
+           "vcs_stream_fields")
+    _wait()
     _check(status.tolist()[0], "vcs_stream_fields (device)")
     return ids, logp
 
 
+@_on_stream
 def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     """Indices of the trainable tokens in order (int32 device tensor)."""
     nt = tok_loss_mask.numel()
@@ -482,15 +527,16 @@ def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     count = _host_words(1, torch.int64)
     nb = vcs_compact_workspace_size(nt)
     ws = _ws(nb, dev)
-    _check(vcs_compact_trainable(tok_loss_mask, nt, idx, cap, count, ws, nb, stream), "vcs_compact_trainable")
+    _check(vcs_compact_trainable(tok_loss_mask, nt, idx, cap, count, ws, nb), "vcs_compact_trainable")
     _check(int(ws[0].item()), "vcs_compact_trainable (device)")
-    _wait(stream)
+    _wait()
     return idx[: count.tolist()[0]]
 
 
+@_on_stream
 def group_advantage(rewards, group_size: int, eps: float = 1e-6, stream=None):
     adv = torch.empty_like(rewards)
-    _check(vcs_group_advantage(rewards, rewards.numel() // group_size, group_size, eps, adv, stream),
+    _check(vcs_group_advantage(rewards, rewards.numel() // group_size, group_size, eps, adv),
            "vcs_group_advantage")
     return adv
 
