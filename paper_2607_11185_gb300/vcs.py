@@ -286,6 +286,13 @@ def _wait():
     torch.cuda.current_stream().synchronize()
 
 
+def _done(status: int, where: str):
+    """Waits for a call whose kernels write pinned host words and checks its status.  One that failed is
+    waited for too: a kernel launched before the failure may still write the words."""
+    _wait()
+    _check(status, where)
+
+
 def _tensors(x):
     if isinstance(x, torch.Tensor):
         yield x
@@ -330,9 +337,8 @@ def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stre
 
 def _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, nb):
     sizes = _host_words(3, torch.int64)   # 24 bytes = vcs_sizes
-    _check(vcs_plan_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, nb),
-           "vcs_plan_segments")
-    _wait()
+    _done(vcs_plan_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, sizes, ws, nb),
+          "vcs_plan_segments")
     ns, nt, tail = sizes.tolist()
     _check(tail >> 32, "vcs_plan_segments (device)")
     return ns, nt, tail & 0xFFFFFFFF
@@ -354,10 +360,9 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
                tok_src_step=torch.empty(nt, dtype=torch.int32, device=dev),
                tok_pos=torch.empty(nt, dtype=torch.int32, device=dev),
                tok_loss_mask=torch.empty(nt, dtype=torch.uint8, device=dev) if with_mask else None)
-    _check(vcs_build_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ns, nt,
-                              out["cu_seqlens"], out["seg_traj"], out["tok_gather"], out["tok_src_step"],
-                              out["tok_pos"], out["tok_loss_mask"], sizes, ws, nb), "vcs_build_segments")
-    _wait()
+    _done(vcs_build_segments(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ns, nt,
+                             out["cu_seqlens"], out["seg_traj"], out["tok_gather"], out["tok_src_step"],
+                             out["tok_pos"], out["tok_loss_mask"], sizes, ws, nb), "vcs_build_segments")
     _check(sizes.tolist()[2] >> 32, "vcs_build_segments (device)")
     out.update(num_segments=ns, num_tokens=nt, max_seqlen=mx)
     return out
@@ -373,9 +378,8 @@ def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
     k = torch.empty((nt, hkv, d), dtype=k_traj.dtype, device=dev)
     v = torch.empty((nt, hkv, d), dtype=v_traj.dtype, device=dev)
     status = _host_words(1, torch.int32)
-    _check(vcs_gather(q_traj, k_traj, v_traj, q_traj.shape[0], tok_gather, nt, hq, hkv, d, q, k, v, status),
-           "vcs_gather")
-    _wait()
+    _done(vcs_gather(q_traj, k_traj, v_traj, q_traj.shape[0], tok_gather, nt, hq, hkv, d, q, k, v, status),
+          "vcs_gather")
     _check(status.tolist()[0], "vcs_gather (device)")
     return q, k, v
 
@@ -418,9 +422,8 @@ def shared_prefix(cu_seqlens, seg_traj, tok_gather, stream=None):
     ns = cu_seqlens.numel() - 1
     out = torch.empty(max(ns, 0), dtype=torch.int32, device=cu_seqlens.device)
     status = _host_words(1, torch.int32)
-    _check(vcs_shared_prefix(cu_seqlens, seg_traj, tok_gather, ns, tok_gather.numel(), out, status),
-           "vcs_shared_prefix")
-    _wait()
+    _done(vcs_shared_prefix(cu_seqlens, seg_traj, tok_gather, ns, tok_gather.numel(), out, status),
+          "vcs_shared_prefix")
     _check(status.tolist()[0], "vcs_shared_prefix (device)")
     return out
 
@@ -510,9 +513,8 @@ def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     ids = torch.empty(nt, dtype=torch.int32, device=dev)
     logp = torch.empty(nt, dtype=torch.float32, device=dev)
     status = _host_words(1, torch.int32)
-    _check(vcs_stream_fields(traj_ids, traj_logp, traj_ids.numel(), tok_gather, tok_loss_mask, nt, ids, logp, status),
-           "vcs_stream_fields")
-    _wait()
+    _done(vcs_stream_fields(traj_ids, traj_logp, traj_ids.numel(), tok_gather, tok_loss_mask, nt, ids, logp, status),
+          "vcs_stream_fields")
     _check(status.tolist()[0], "vcs_stream_fields (device)")
     return ids, logp
 
@@ -527,9 +529,8 @@ def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     count = _host_words(1, torch.int64)
     nb = vcs_compact_workspace_size(nt)
     ws = _ws(nb, dev)
-    _check(vcs_compact_trainable(tok_loss_mask, nt, idx, cap, count, ws, nb), "vcs_compact_trainable")
+    _done(vcs_compact_trainable(tok_loss_mask, nt, idx, cap, count, ws, nb), "vcs_compact_trainable")
     _check(int(ws[0].item()), "vcs_compact_trainable (device)")
-    _wait()
     return idx[: count.tolist()[0]]
 
 

@@ -124,3 +124,27 @@ def test_workspace_of_a_running_call_is_not_handed_out(monkeypatch):
     assert not side.query()
     torch.cuda.synchronize()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("name", ["plan_segments", "build_segments", "gather", "shared_prefix", "stream_fields",
+                                  "compact_trainable"])
+def test_failed_call_is_waited_for(name, monkeypatch):
+    # a call that launched a kernel and then failed: its pinned words stay until the kernel is done
+    from paper_2607_11185_gb300 import vcs
+    x = inputs()
+    lay = vcs.build_segments(*x[:3], 2, 1)
+    gat, mask = lay["tok_gather"], lay["tok_loss_mask"]
+    args = dict(plan_segments=(*x[:3], 2, 1), build_segments=(*x[:3], 2, 1), gather=(*x[3:], gat),
+                shared_prefix=(lay["cu_seqlens"], lay["seg_traj"], gat),
+                stream_fields=(gat, gat.float(), gat, mask), compact_trainable=(mask,))[name]
+    real = getattr(vcs, "vcs_" + name)
+
+    def fails(*a, **kw):
+        torch.cuda._sleep(BUSY)
+        assert real(*a, **kw) == 0
+        return 5
+
+    monkeypatch.setattr(vcs, "vcs_" + name, fails)
+    with pytest.raises(vcs.VcsError):
+        getattr(vcs, name)(*args)
+    assert torch.cuda.current_stream().query()
