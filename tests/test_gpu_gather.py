@@ -112,3 +112,26 @@ def test_row_sizes_around_the_warp(hq, hkv, d, with_kv):
     assert int(st.item()) == 0
     for src, got in zip((q, k, v)[:3 if with_kv else 1], out):
         assert torch.equal(got, src[idx.long()])
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4864, 4865, 160000])
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 8), (1, 3, 16), (7, 1, 72), (127, 1, 8), (127, 127, 8), (128, 1, 8),
+                                      (1, 128, 8)])
+def test_narrow_rows(hq, hkv, d, n):
+    # rows of 1 .. 128 chunks around the width at which a warp takes one token, token counts around one
+    # step, one warp's tokens and one pass of the grid; indices out of range skip their rows alone
+    from paper_2607_11185_gb300 import vcs
+    g = torch.Generator(device="cuda").manual_seed(n + hq)
+    src = [torch.randn((333, h, d), generator=g, device="cuda").bfloat16() for h in (hq, hkv, hkv)]
+    idx = torch.randint(0, 333, (n,), generator=g, device="cuda", dtype=torch.int32)
+    bad = torch.rand(n, generator=g, device="cuda") < 0.01
+    bad[n - 1] = True
+    idx[bad] = torch.where(torch.rand(n, generator=g, device="cuda") < 0.5, -1, 333).int()[bad]
+    out = [torch.full((n, h, d), 7.0, dtype=torch.bfloat16, device="cuda") for h in (hq, hkv, hkv)]
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert vcs.vcs_gather(*src, 333, idx, n, hq, hkv, d, *out, st) == 0
+    assert int(st.item()) == 6
+    for x, got in zip(src, out):
+        want = torch.where(bad[:, None, None], torch.tensor(7.0, dtype=torch.bfloat16, device="cuda"),
+                           x[idx.clamp(0, 332).long()])
+        assert torch.equal(got, want)
