@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(kThreads) grpo_loss_tokens(const __grid_consta
   if (threadIdx.x == 0) *a.loss = total * a.inv_ntraj64;
 }
 
-// one warp per group: mean and population standard deviation in double (one group of 8: 8.9 us with
-// events around the call, nearly all of it the launch; 10.9 with a thread per group)
-__global__ void __launch_bounds__(256) group_advantage_kernel(const float* __restrict__ rewards, int64_t num_groups,
+// Mean and population standard deviation in double.  One warp per group: a group's latency (one group of
+// 8: 8.9 us with events around the call, nearly all of it the launch; 10.9 with a thread per group).
+__global__ void __launch_bounds__(256) group_advantage_warp(const float* __restrict__ rewards, int64_t num_groups,
                                                               int32_t group_size, float eps, float* __restrict__ adv) {
   const int lane = threadIdx.x & 31;
   auto warp_sum = [](double x) {
@@ -177,6 +177,25 @@ __global__ void __launch_bounds__(256) group_advantage_kernel(const float* __res
     }
     const double den = sqrt(warp_sum(var) / group_size) + (double)eps;
     for (int j = lane; j < group_size; j += 32) adv[gi * group_size + j] = (float)((r[j] - mean) / den);
+  }
+}
+
+// One thread per group: every lane's double arithmetic, which bounds many groups, is another group's.
+__global__ void group_advantage_thread(const float* __restrict__ rewards, int64_t num_groups, int32_t group_size,
+                                       float eps, float* __restrict__ adv) {
+  for (int64_t gi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gi < num_groups;
+       gi += (int64_t)gridDim.x * blockDim.x) {
+    const float* r = rewards + gi * group_size;
+    double mean = 0.0;
+    for (int j = 0; j < group_size; ++j) mean += r[j];
+    mean /= group_size;
+    double var = 0.0;
+    for (int j = 0; j < group_size; ++j) {
+      const double d = r[j] - mean;
+      var += d * d;
+    }
+    const double den = sqrt(var / group_size) + (double)eps;
+    for (int j = 0; j < group_size; ++j) adv[gi * group_size + j] = (float)((r[j] - mean) / den);
   }
 }
 
@@ -232,9 +251,15 @@ cudaError_t launch_grpo_loss(const float* logp, const float* old_logp, const flo
 cudaError_t launch_group_advantage(const float* rewards, int64_t num_groups, int32_t group_size, float eps,
                                    float* adv, cudaStream_t st) {
   if (num_groups == 0) return cudaSuccess;
-  int64_t blocks = (num_groups + 7) / 8;
+  // Measured up to 1 M groups: a warp a group takes 1.8 + 1.1 ceil(group_size / 32) ns a group, a thread a
+  // group 1,140 ns a member until the groups fill the chip, so the line is where the two are equal (8 a
+  // group, us, warp / thread: 12 / 16 at 2,048 groups, 20 / 16 at 4,096, 2,950 / 295 at 1 M).  Past 512
+  // members a warp, whose loads are whole lines, is no slower at any count (32,768 of 1,024: 1,120 / 1,165).
+  const bool thread = group_size <= 512 && num_groups >= 11400ll * group_size / (18 + 11 * ((group_size + 31) / 32));
+  int64_t blocks = thread ? (num_groups + 255) / 256 : (num_groups + 7) / 8;
   if (blocks > 152 * 8) blocks = 152 * 8;
-  group_advantage_kernel<<<(unsigned)blocks, 256, 0, st>>>(rewards, num_groups, group_size, eps, adv);
+  (thread ? group_advantage_thread : group_advantage_warp)<<<(unsigned)blocks, 256, 0, st>>>(rewards, num_groups,
+                                                                                            group_size, eps, adv);
   return cudaGetLastError();
 }
 

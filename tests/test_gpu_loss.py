@@ -210,3 +210,19 @@ def test_sizes_and_alignments(n, shift):
                              0.28, 3.0, 1e-4, loss, dl, ws, nb) == 0
     assert int(ws[:4].view(torch.int32).item()) == 0
     _tol_check(float(loss.item()), dl.cpu().numpy().astype(np.float64), logp, old, ref, mask, cu, st, adv, 3)
+
+
+@pytest.mark.parametrize("group_size", [1, 2, 8, 32, 33, 64, 512, 513])
+def test_group_advantage_around_the_line_between_its_kernels(group_size):
+    # from this many groups on a thread takes a group (up to 512 members), below it a warp; a sum in
+    # another order differs by group_size roundings of double, far below fp32's
+    from paper_2607_11185_gb300 import vcs
+    line = -(-11400 * group_size // (18 + 11 * ((group_size + 31) // 32)))
+    for n in (line - 1, line, line + 257):
+        g = torch.Generator(device=DEV).manual_seed(n)
+        r = torch.rand((n, group_size), generator=g, device=DEV)
+        r[::3] = 0.25  # groups without spread: 0
+        got = vcs.group_advantage(r.reshape(-1), group_size).reshape(n, group_size).double()
+        x = r.double()
+        want = (x - x.mean(1, keepdim=True)) / (x.std(1, correction=0, keepdim=True) + 1e-6)
+        assert (got - want).abs().max() <= 1e-6 * max(1.0, float(want.abs().max()))
