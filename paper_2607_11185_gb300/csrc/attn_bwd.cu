@@ -226,8 +226,9 @@ static_assert(sizeof(BwdBars) <= Bwd<64>::BAR_BYTES && sizeof(BwdBars) <= Bwd<12
 // warp's query i and whether its values are added (else 0 is).  Four reductions (16 lines of 128
 // bytes) a warp every 200 cycles: 1.268 ms (14/2/64, 16 segments of 4,096) against 1.293 at full
 // speed and 1.273 and 1.288 with 300 and 400.
+// Groups of 8 rows from `rows` on, past the segment's end, are left out.
 template <typename RowFn>
-__device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, RowFn row) {
+__device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, int rows, RowFn row) {
   const bool odd = lane & 1, oddr = lane & 4;
   const uint32_t t0 = clock();
   const int coff = (lane & 1) * 8 + ((lane >> 1) & 1) * 4 + (oddr ? 16 : 0);
@@ -235,6 +236,7 @@ __device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, 
   for (int g = 0; g < 2; ++g)
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
+      if (16 * g + 8 * half >= rows) return;
       const int rr = 16 * g + 8 * half + ((lane >> 2) & 6);
       bool le, lo;
       float* pe = row(rr, le);
@@ -780,7 +782,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     if (ok) ok = mbar_wait_warp(&bars->acc_done, 0);
     if (!ok) {
       abort_now();
-    } else {
+    } else if (n * C::BM + quad * 32 < L) {  // the warp has rows in the segment
       tc_fence_after();
       // warpgroup 1 writes dK, warpgroup 2 writes dV (key row r on the TMEM lane)
       const uint32_t col = k == 0 ? C::TM_DK : C::TM_DV;
@@ -888,7 +890,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         // 16 reductions a warp, then a pause until 20 cycles have passed for each: issued as fast as
         // the SM takes them (22 cycles each) they hold up the compute warps' shared-memory accesses.
         // No branch per reduction (it would double the kernel's time): rows past the segment end, and
-        // gather indices out of range, add 0 to a row in range.
+        // gather indices out of range, add 0 to a row in range; a burst wholly past the end is left out.
         const uint32_t t0 = clock();
         auto burst = [&](int c, auto add) {
 #pragma unroll
@@ -923,6 +925,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         } else if constexpr (GATHER) {
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
+            if (16 * c >= qn) break;
             const unsigned lives = __ballot_sync(0xffffffffu, live[c / 2]);
             burst(c, [&](int q) {
               const int t = __shfl_sync(0xffffffffu, tok[q / 32], q % 32);
@@ -931,10 +934,12 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           }
         } else {
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
+          for (int c = 0; c < 8; ++c) {
+            if (16 * c >= qn) break;
             burst(c, [&](int q) {
               red_add(base + min(q, qn - 1) * row_stride, q < qn ? __uint_as_float(v[q]) : 0.f);
             });
+          }
         }
       } else {
         uint32_t v[2][32];
@@ -951,13 +956,13 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           const bool live = qr + lane < qn && tok >= 0 && tok < traj_tokens;
           if (tok < 0 || tok >= traj_tokens) tok = 0;
           const unsigned lives = __ballot_sync(0xffffffffu, live);
-          drain_d64(v, lane, [&](int i, bool& l) -> float* {
+          drain_d64(v, lane, qn - qr, [&](int i, bool& l) -> float* {
             l = (lives >> i) & 1;
             return base + (size_t)__shfl_sync(0xffffffffu, tok, i) * row_stride;
           });
         } else {
           base += (size_t)(start + q0) * row_stride;
-          drain_d64(v, lane, [&](int i, bool& l) -> float* {
+          drain_d64(v, lane, qn - qr, [&](int i, bool& l) -> float* {
             l = qr + i < qn;
             return base + min(qr + i, qn - 1) * row_stride;
           });

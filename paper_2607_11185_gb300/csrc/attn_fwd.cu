@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (ok) ok = mbar_wait_warp(&bars->o_done[wg], C::OWN_P ? mt & 1 : 0);
       if (!ok) {
         on_timeout(bars, status);
-      } else {
+      } else if (mt * C::BM + quad * 32 < L) {  // the warp has rows in the segment
         tc_fence_after();
         const int row = mt * C::BM + r;
         const bool valid = row < L;

@@ -255,3 +255,25 @@ def test_dk_dv_summed_in_query_order_d64():
     assert 8 < want[0].sum() < d - 8 and 8 < want[1].sum() < d - 8  # both outcomes occur
     assert np.array_equal(dk[0, 0, 1:].float().cpu().numpy(), want[0, 1:])
     assert np.array_equal(dv[0, 0, 1:].float().cpu().numpy(), want[1, 1:])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_segment_ends_around_the_drains_row_groups(d):
+    """The last query tile's rows past the segment end are left out of the dQ reductions 8 (d = 64) or 16
+    (d = 128) at a time, and warps without rows skip the epilogue: ends on both sides of each, against
+    the oracle, and the gathered backward (rows in trajectory order) against the same gradients."""
+    from paper_2607_11185_gb300 import vcs
+    lengths = [1, 7, 8, 9, 15, 16, 17, 24, 25, 31, 32, 33, 48, 49, 64, 65, 96, 97, 112, 113, 120, 121, 127, 128, 129,
+               144, 145, 161, 256 + 33]
+    cu = cu_from_lengths(lengths)
+    q, k, v, do = workloads.draw_dense(77 + d, int(cu[-1]), 2, 1, d, device="cuda")
+    o, lse, *grads = run(q, k, v, do, cu)
+    want = oatt.attn_bwd(q.cpu(), k.cpu(), v.cpu(), do.cpu(), cu)
+    for s, e in zip(cu, cu[1:]):
+        for name, got, ref in zip(("dq", "dk", "dv"), grads, want):
+            # a segment of a few rows averages few bf16 roundings
+            assert rel_err(got[s:e].float().cpu().numpy(), ref[s:e]) <= 2.5 * REL, (name, e - s)
+    gat = torch.arange(int(cu[-1]), dtype=torch.int32, device="cuda")
+    got = vcs.attn_bwd_gathered(q, k, v, gat, o, lse, do, torch.from_numpy(cu).cuda(), max(lengths))
+    for name, a, b in zip(("dq", "dk", "dv"), got, grads):
+        assert (a.double() - b.double()).norm() <= 5e-3 * b.double().norm(), name
