@@ -48,8 +48,8 @@
 // the last tile, whose S(j+1) completing means their reads are done.  (The
 // gathered variant, whose producer issues its loads more slowly, has them
 // handed back by commits as soon as the MMAs are done.)  The ring order puts
-// the two tiles step j reads, K_{j+1} and V_j, next to each other, so the
-// tiled loads complete one barrier per step and the MMA thread waits once a
+// the two tiles step j reads, K_{j+1} and V_j, next to each other, so they
+// complete one barrier per step and the MMA thread waits once a
 // step for its K/V, at the top of the step.
 //
 // d = 64: the MMAs of a step take about 1,020 cycles and the softmax warps bound it, so
@@ -90,7 +90,7 @@ struct Fwd {
   static constexpr int BLOCK = BM * 128;            // bytes of one 128 x 64 column block
   static constexpr bool OWN_P = D == 64;            // P in TMEM columns of its own
   static constexpr int NSLOT = OWN_P ? 8 : 5;
-  static constexpr int NGRP = 4;                    // ring-item group barriers (tiled loads)
+  static constexpr int NGRP = 4;                    // ring-item group barriers
   static constexpr int OFF_Q0 = 0;
   static constexpr int OFF_Q1 = TILE;
   static constexpr int OFF_KV = 2 * TILE;
@@ -105,9 +105,9 @@ static_assert(Fwd<128>::SMEM <= 232448, "shared memory budget");
 
 struct Bars {
   uint64_t q_full;
-  uint64_t kv_full[8];   // per ring slot (gathered loads, OWN_P)
+  uint64_t kv_full[8];   // per ring slot (OWN_P)
   uint64_t kv_empty[8];
-  uint64_t grp_full[4];  // per pair of ring items consumed in one step (tiled loads without OWN_P)
+  uint64_t grp_full[4];  // per pair of ring items consumed in one step (without OWN_P)
   uint64_t s_full[2];
   uint64_t s_read[2];    // OWN_P: S(j) is in the softmax warps' registers
   uint64_t p_full[2];
@@ -339,6 +339,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     setmaxnreg_dec<kRegCtrl>();
     if (warp == 0 && (GATHER || lane == 0)) {
     // ------------------------------------------------------------ producer
+      // Without OWN_P items 2m-1, 2m (K_m, V_{m-1}) are the ones step m-1 consumes: they complete one
+      // barrier, armed for both by the first; group 0 (K_0) and group nkv (V_{nkv-1}) hold one item
+      auto item_bar = [&](int c) -> uint64_t* {
+        return C::OWN_P ? &bars->kv_full[c % C::NSLOT] : &bars->grp_full[((c + 1) >> 1) % C::NGRP];
+      };
+      auto arm_item = [&](int c) {
+        const int m = (c + 1) >> 1;
+        if (C::OWN_P)
+          mbar_arrive_expect_tx(item_bar(c), C::TILE);
+        else if (c == 0 || (c & 1))
+          mbar_arrive_expect_tx(item_bar(c), (m == 0 || m == nkv ? 1 : 2) * C::TILE);
+      };
       if constexpr (GATHER) {
         // the whole warp: lane 0 posts each tile's bytes and waits for free slots
         if (lane == 0) {
@@ -357,6 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const bool is_v = c == 2 * nkv - 1 || (c > 0 && (c & 1) == 0);
           const int j = c == 2 * nkv - 1 ? nkv - 1 : (is_v ? (c - 2) >> 1 : (c + 1) >> 1);
           const int slot = c % C::NSLOT, round = c / C::NSLOT;
+          uint64_t* gb = item_bar(c);
           int go = 1;
           if (lane == 0) {
             if (c >= C::NSLOT && !mbar_wait(&bars->kv_empty[slot], (round - 1) & 1)) {
@@ -365,12 +378,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             } else if (aborted(bars)) {
               go = 0;
             } else {
-              mbar_arrive_expect_tx(&bars->kv_full[slot], C::TILE);
+              arm_item(c);
             }
           }
           if (!__shfl_sync(0xffffffffu, go, 0)) break;
           load_traj_tile<C::KB, C::BLOCK>(smem + C::OFF_KV + slot * C::TILE, is_v ? &tm_v : &tm_k,
-                                          is_v ? &tm_vr : &tm_kr, is_v ? &tm_vs : &tm_ks, &bars->kv_full[slot], g, D, start + j * C::BN,
+                                          is_v ? &tm_vr : &tm_kr, is_v ? &tm_vs : &tm_ks, gb, g, D, start + j * C::BN,
                                           end - 1, tok_gather, traj_tokens, status, lane);
         }
       } else {
@@ -395,15 +408,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           if (aborted(bars)) break;
-          // items 2m-1, 2m (K_m, V_{m-1}) are the ones step m-1 consumes: they complete one
-          // barrier, armed for both by the first; group 0 (K_0) and group nkv (V_{nkv-1})
-          // hold one item
-          const int m = (c + 1) >> 1;
-          uint64_t* gb = C::OWN_P ? &bars->kv_full[slot] : &bars->grp_full[m % C::NGRP];
-          if (C::OWN_P)
-            mbar_arrive_expect_tx(gb, C::TILE);
-          else if (c == 0 || (c & 1))
-            mbar_arrive_expect_tx(gb, (m == 0 || m == nkv ? 1 : 2) * C::TILE);
+          uint64_t* gb = item_bar(c);
+          arm_item(c);
           const CUtensorMap* tm = is_v ? &tm_v : &tm_k;
 #pragma unroll
           for (int kb = 0; kb < C::KB; ++kb)
@@ -453,7 +459,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The whole warp runs the loop and one elected lane issues, so that descriptors and addresses
     // stay in uniform registers; as a one-lane branch each MMA took 75-100 cycles to issue instead of
     // the 64 it executes in (four segments of 8,192 at 40/8/128: 1.774 -> 1.674 ms, sixteen of 4,096
-    // at 14/2/64: 0.618 -> 0.562).  As above, no lane's answer decides where the warp goes.
+    // at 14/2/64: 0.618 -> 0.562).  As above, no lane's answer decides where the
+    // warp goes; here a vote a step does, behind the wait for K and V (waits that end in a branch on the
+    // lane's own state cost the gathered form 3%, a vote on each wait 5%).  Gathered loads used to
+    // complete a barrier per ring item: 28/4/128, eight segments of 4,096, 0.713 -> 0.705 ms.
       bool ok = mbar_wait(&bars->q_full, 0);
       // descriptors built once; the issue loops only add compile-time offsets
       const uint64_t q0d = smem_desc(sbase + C::OFF_Q0, 16, 1024), q1d = desc_at(q0d, C::TILE);
@@ -464,15 +473,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto v_item = [&](int j) { return j == nkv - 1 ? 2 * nkv - 1 : 2 * j + 2; };
       auto k_off = [&](int j) { return (uint32_t)((k_item(j) % C::NSLOT) * C::TILE); };
       auto v_off = [&](int j) { return (uint32_t)((v_item(j) % C::NSLOT) * C::TILE); };
-      // tiled loads: group m holds K_m and V_{m-1} (group 0 only K_0, group nkv only
-      // V_{nkv-1}); gathered loads: one barrier per ring item
+      // group m holds K_m and V_{m-1} (group 0 only K_0, group nkv only V_{nkv-1})
       auto acquire_group = [&](int m) {
-        if constexpr (GATHER) {
-          if (m < nkv) ok = ok && mbar_wait(&bars->kv_full[k_item(m) % C::NSLOT], (k_item(m) / C::NSLOT) & 1);
-          if (m > 0) ok = ok && mbar_wait(&bars->kv_full[v_item(m - 1) % C::NSLOT], (v_item(m - 1) / C::NSLOT) & 1);
-        } else {
-          ok = ok && mbar_wait(&bars->grp_full[m % C::NGRP], (m / C::NGRP) & 1);
-        }
+        ok &= mbar_wait(&bars->grp_full[m % C::NGRP], (m / C::NGRP) & 1);
         tc_fence_after();
       };
       uint32_t kaddr = k_off(0), vaddr = 0;  // slot byte offsets of K_{j+1} and V_j
@@ -494,11 +497,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int j = 0; j < nkv; ++j) {
         const bool next = j + 1 < nkv;
         acquire_group(j + 1);
+        if (!__all_sync(0xffffffffu, ok)) break;
         vaddr = v_off(j);
         if (next) kaddr = k_off(j + 1);
         // tile 0: O0 += P0(j) V_j, then S0(j+1)
         if (j <= m0) {
-          ok = ok && mbar_wait(&bars->p_full[0], j & 1);
+          ok &= mbar_wait(&bars->p_full[0], j & 1);
           tc_fence_after();
           if (elect_one() && ok) {
             issue_pv<D>(tmem + C::TM_O0, tmem + C::TM_S0, desc_at(kv_mnmaj, vaddr), j > 0);
@@ -513,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         // tile 1
         if (has1) {
-          ok = ok && mbar_wait(&bars->p_full[1], j & 1);
+          ok &= mbar_wait(&bars->p_full[1], j & 1);
           tc_fence_after();
           if (elect_one() && ok) {
             issue_pv<D>(tmem + C::TM_O1, tmem + C::TM_S1, desc_at(kv_mnmaj, vaddr), j > 0);
