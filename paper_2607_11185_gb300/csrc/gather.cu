@@ -31,8 +31,9 @@ __device__ __forceinline__ void st_stream(int4* p, int4 v) {
 }
 
 // Copies chunks lane, lane + 32, ... of a row, kUnroll loads in flight per lane.
-__device__ __forceinline__ void copy_row(const int4* __restrict__ src, int4* __restrict__ dst, int chunks, int lane) {
-  int c = lane;
+template <typename Chunk>
+__device__ __forceinline__ void copy_row(const int4* __restrict__ src, int4* __restrict__ dst, Chunk chunks, int lane) {
+  Chunk c = lane;
   for (; c + 32 * (kUnroll - 1) < chunks; c += 32 * kUnroll) {
     int4 v[kUnroll];
 #pragma unroll
@@ -43,14 +44,17 @@ __device__ __forceinline__ void copy_row(const int4* __restrict__ src, int4* __r
   for (; c < chunks; c += 32) st_stream(dst + c, ld_stream(src + c));
 }
 
-// One warp per segment token, for rows of at least kNarrow chunks: its Q, K and V rows in one launch.  The token's index is loaded a token
-// ahead; per row there is no division and one address each (a chunk-per-thread form with a 64-bit
-// division per chunk, launched once per tensor, took 1.19 ms for the 3.5 GB of a long-horizon rollout,
-// this form 1.06: 6.7 TB/s read and written; 8 loads in flight a lane 1.12).
+// One warp per segment token, for rows of at least kNarrow chunks: its Q, K and V rows in one launch.
+// The token's index is loaded a token ahead; per row there is no division and one address each (a
+// chunk-per-thread form with a 64-bit division per chunk, launched once per tensor, took 1.19 ms for
+// the 3.5 GB of a long-horizon rollout, this form 1.06: 6.7 TB/s read and written; 8 loads in flight a
+// lane 1.12).  Chunk: int, or int64_t for rows of 2^30 chunks and more (1.2 M tokens at 8/2/128 take
+// 1,200 us with it, 1,116 with int).
+template <typename Chunk>
 __global__ void __launch_bounds__(kThreads)
     gather_rows(const int4* __restrict__ q_src, const int4* __restrict__ k_src, const int4* __restrict__ v_src,
-                int64_t traj_tokens, const int32_t* __restrict__ tok_gather, int64_t num_tokens, int q_chunks,
-                int kv_chunks, int4* __restrict__ q, int4* __restrict__ k, int4* __restrict__ v, int32_t* status) {
+                int64_t traj_tokens, const int32_t* __restrict__ tok_gather, int64_t num_tokens, Chunk q_chunks,
+                Chunk kv_chunks, int4* __restrict__ q, int4* __restrict__ k, int4* __restrict__ v, int32_t* status) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
   int64_t n = blockIdx.x * (int64_t)(kThreads / 32) + (threadIdx.x >> 5);
@@ -77,7 +81,8 @@ __global__ void __launch_bounds__(kThreads)
 // 8 dims 34.8 / 393 / 28.7, 1/1/64 190 / 446 / 170, 14/2/64 1,001 / 1,114 / 971.  From kNarrow chunks on a
 // warp a token is the faster (8/2/128: 1,364 / 1,116 / 1,288; 28/4/128: 3,829 / 3,331 / 3,762).
 constexpr int kNarrow = 128;
-constexpr int kMagicShift = 24;  // chunk f of a run of rows of c is row f * (2^24 / c + 1) >> 24: exact for f < 2^24 / c
+// chunk f of a run of rows of c chunks lies in row f * (2^24 / c + 1) >> 24, exactly for f < 2^24 / c
+constexpr int kMagicShift = 24;
 static_assert((32 * kNarrow + 32) * kNarrow <= 1 << kMagicShift, "row of a chunk");
 
 template <int UNROLL>
@@ -126,7 +131,6 @@ cudaError_t launch_gather(const void* q_src, const void* k_src, const void* v_sr
                           const int32_t* tok_gather, int64_t num_tokens, int64_t q_row_bytes, int64_t kv_row_bytes,
                           void* q, void* k, void* v, int32_t* dev_status, cudaStream_t st) {
   if (num_tokens == 0) return cudaSuccess;
-  if (q_row_bytes / 16 > INT32_MAX || kv_row_bytes / 16 > INT32_MAX) return cudaErrorInvalidValue;
   const int64_t cap = 152 * 16;
   const int64_t q_chunks = q_row_bytes / 16, kv_chunks = kv_row_bytes / 16;
   if (q_chunks < kNarrow && kv_chunks < kNarrow) {
@@ -138,7 +142,7 @@ cudaError_t launch_gather(const void* q_src, const void* k_src, const void* v_sr
     int64_t blocks = (warps + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > cap) blocks = cap;
     auto magic = [](int64_t c) { return c > 0 ? (1u << kMagicShift) / (uint32_t)c + 1 : 0u; };
-    // of a few steps a pass none waits for another, and more warps fit (Q alone, one chunk a row: 20.5 -> 16.4 us)
+    // of a few steps a pass none waits for another, and more warps fit (Q alone, a chunk a row: 20.5 -> 16.4 us)
     const auto kernel = q_chunks + 2 * kv_chunks < kUnroll ? gather_narrow<1> : gather_narrow<kUnroll>;
     kernel<<<(unsigned)blocks, kThreads, 0, st>>>(
         static_cast<const int4*>(q_src), static_cast<const int4*>(k_src), static_cast<const int4*>(v_src), traj_tokens,
@@ -148,10 +152,16 @@ cudaError_t launch_gather(const void* q_src, const void* k_src, const void* v_sr
   }
   int64_t blocks = (num_tokens + kThreads / 32 - 1) / (kThreads / 32);
   if (blocks > cap) blocks = cap;
-  gather_rows<<<(unsigned)blocks, kThreads, 0, st>>>(
-      static_cast<const int4*>(q_src), static_cast<const int4*>(k_src), static_cast<const int4*>(v_src), traj_tokens,
-      tok_gather, num_tokens, (int)(q_row_bytes / 16), (int)(kv_row_bytes / 16), static_cast<int4*>(q),
-      static_cast<int4*>(k), static_cast<int4*>(v), dev_status);
+  auto launch = [&](auto kernel, auto qc, auto kvc) {
+    kernel<<<(unsigned)blocks, kThreads, 0, st>>>(
+        static_cast<const int4*>(q_src), static_cast<const int4*>(k_src), static_cast<const int4*>(v_src), traj_tokens,
+        tok_gather, num_tokens, qc, kvc, static_cast<int4*>(q), static_cast<int4*>(k), static_cast<int4*>(v),
+        dev_status);
+  };
+  if (q_chunks < 1 << 30 && kv_chunks < 1 << 30)
+    launch(gather_rows<int>, (int)q_chunks, (int)kv_chunks);
+  else
+    launch(gather_rows<int64_t>, q_chunks, kv_chunks);
   return cudaGetLastError();
 }
 

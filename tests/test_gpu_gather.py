@@ -135,3 +135,13 @@ def test_narrow_rows(hq, hkv, d, n):
         want = torch.where(bad[:, None, None], torch.tensor(7.0, dtype=torch.bfloat16, device="cuda"),
                            x[idx.clamp(0, 332).long()])
         assert torch.equal(got, want)
+
+
+def test_rows_of_more_chunks_than_an_int32():
+    # 2^28 heads of 128 dims, 64 GB a row: taken, and rows without a source are skipped without a touch
+    from paper_2607_11185_gb300 import vcs
+    buf = torch.zeros(8, dtype=torch.bfloat16, device="cuda")
+    idx = torch.tensor([-1, 1], dtype=torch.int32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert vcs.vcs_gather(buf, None, None, 1, idx, 2, 1 << 28, 1, 128, buf, None, None, st) == 0
+    assert int(st.item()) == 6
