@@ -226,9 +226,10 @@ static_assert(sizeof(BwdBars) <= Bwd<64>::BAR_BYTES && sizeof(BwdBars) <= Bwd<12
 // warp's query i and whether its values are added (else 0 is).  Four reductions (16 lines of 128
 // bytes) a warp every 200 cycles: 1.268 ms (14/2/64, 16 segments of 4,096) against 1.293 at full
 // speed and 1.273 and 1.288 with 300 and 400.
-// Groups of 8 rows from `rows` on, past the segment's end, are left out.
+// Rows past the segment's end add 0 as well: leaving groups of them out put a branch between the
+// reductions that cost full tiles 8% (1.255 -> 1.356 ms).
 template <typename RowFn>
-__device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, int rows, RowFn row) {
+__device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, RowFn row) {
   const bool odd = lane & 1, oddr = lane & 4;
   const uint32_t t0 = clock();
   const int coff = (lane & 1) * 8 + ((lane >> 1) & 1) * 4 + (oddr ? 16 : 0);
@@ -236,7 +237,6 @@ __device__ __forceinline__ void drain_d64(const uint32_t (&v)[2][32], int lane, 
   for (int g = 0; g < 2; ++g)
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
-      if (16 * g + 8 * half >= rows) return;
       const int rr = 16 * g + 8 * half + ((lane >> 2) & 6);
       bool le, lo;
       float* pe = row(rr, le);
@@ -956,13 +956,13 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
           const bool live = qr + lane < qn && tok >= 0 && tok < traj_tokens;
           if (tok < 0 || tok >= traj_tokens) tok = 0;
           const unsigned lives = __ballot_sync(0xffffffffu, live);
-          drain_d64(v, lane, qn - qr, [&](int i, bool& l) -> float* {
+          drain_d64(v, lane, [&](int i, bool& l) -> float* {
             l = (lives >> i) & 1;
             return base + (size_t)__shfl_sync(0xffffffffu, tok, i) * row_stride;
           });
         } else {
           base += (size_t)(start + q0) * row_stride;
-          drain_d64(v, lane, qn - qr, [&](int i, bool& l) -> float* {
+          drain_d64(v, lane, [&](int i, bool& l) -> float* {
             l = qr + i < qn;
             return base + min(qr + i, qn - 1) * row_stride;
           });

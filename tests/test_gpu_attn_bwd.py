@@ -259,9 +259,9 @@ def test_dk_dv_summed_in_query_order_d64():
 
 @pytest.mark.parametrize("d", [64, 128])
 def test_segment_ends_around_the_drains_row_groups(d):
-    """The last query tile's rows past the segment end are left out of the dQ reductions 8 (d = 64) or 16
-    (d = 128) at a time, and warps without rows skip the epilogue: ends on both sides of each, against
-    the oracle, and the gathered backward (rows in trajectory order) against the same gradients."""
+    """At d = 128 the last query tile's rows past the segment end are left out of the dQ reductions 16 at a
+    time, and warps without rows skip the epilogue: ends on both sides of each, against the oracle, and
+    the gathered backward (rows in trajectory order) against the same gradients."""
     from paper_2607_11185_gb300 import vcs
     lengths = [1, 7, 8, 9, 15, 16, 17, 24, 25, 31, 32, 33, 48, 49, 64, 65, 96, 97, 112, 113, 120, 121, 127, 128, 129,
                144, 145, 161, 256 + 33]
