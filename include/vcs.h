@@ -23,6 +23,9 @@
  *     vcs_status into a device-visible int32 status word named by each call;
  *     the offending work is skipped, never trapped.  The caller reads that
  *     word after synchronising.
+ *   - A word called device-visible below lies in device memory or in pinned
+ *     (mapped) host memory, which the host reads after synchronising without
+ *     a copy.  It must stay allocated until the call's work is done.
  *   - Counts of tokens, steps and segments are limited to INT32_MAX.
  *
  * Step model (the readings of the paper that the layout follows):
@@ -127,7 +130,7 @@ vcs_status vcs_build_segments(const int32_t* cu_steps, int32_t num_traj, int64_t
  *   q_traj [traj_tokens, hq, d], k_traj / v_traj [traj_tokens, hkv, d] bf16 device
  *   tok_gather [num_tokens] int32 device (from vcs_build_segments)
  *   q [num_tokens, hq, d], k / v [num_tokens, hkv, d] bf16 device outputs
- *   dev_status  int32 device word or NULL: set to VCS_ERR_DEVICE_CHECK if a
+ *   dev_status  int32 device-visible word or NULL: set to VCS_ERR_DEVICE_CHECK if a
  *               gather index is outside [0, traj_tokens) (that row is skipped)
  * k_traj/v_traj/k/v may all be NULL to gather Q only.  Bit-exact copy.
  * ------------------------------------------------------------------------ */
@@ -278,7 +281,7 @@ vcs_status vcs_attn_bwd_gathered(const void* q_traj, const void* k_traj, const v
  * seg_traj[s] != seg_traj[s-1] or s = 0.
  *   cu_seqlens, seg_traj, tok_gather  from vcs_build_segments (device)
  *   seg_shared  int32 [num_segments] device (written)
- *   dev_status  int32 device word or NULL: VCS_ERR_DEVICE_CHECK for
+ *   dev_status  int32 device-visible word or NULL: VCS_ERR_DEVICE_CHECK for
  *               inconsistent cu_seqlens (that segment gets 0)
  *
  * vcs_attn_fwd_reuse: vcs_attn_fwd's result (bit for bit) with seg_shared
@@ -314,7 +317,7 @@ vcs_status vcs_attn_fwd_reuse(const void* q, const void* k, const void* v, const
  *              trajectories' tokens (read only for response tokens)
  *   tok_gather, tok_loss_mask  from vcs_build_segments
  *   ids, logp  int32 / fp32 [num_tokens] device (written)
- *   dev_status int32 device word or NULL: VCS_ERR_DEVICE_CHECK when a gather
+ *   dev_status int32 device-visible word or NULL: VCS_ERR_DEVICE_CHECK when a gather
  *              index is outside [0, traj_tokens) (that token gets 0, 0)
  * Returns VCS_ERR_INVALID_ARG for a negative count or a null pointer,
  * VCS_ERR_OVERFLOW for counts above INT32_MAX.
@@ -328,7 +331,7 @@ vcs_status vcs_stream_fields(const int32_t* traj_ids, const float* traj_logp, in
  * App. C.1).
  *   idx        int32 [idx_capacity] device (written: the first min(count,
  *              idx_capacity) entries)
- *   count      int64 device, 1 value (written): the number of trainable tokens
+ *   count      int64 device-visible, 1 value (written): the number of trainable tokens
  *   ws         device workspace of vcs_compact_workspace_size(num_tokens) bytes,
  *              256-byte aligned; its first int32 is the device status word
  *              (VCS_ERR_CAPACITY when count > idx_capacity)
@@ -401,7 +404,7 @@ vcs_status vcs_group_advantage(const float* rewards, int64_t num_groups, int32_t
  * VCS_ERR_DEVICE_TIMEOUT into *dev_status.  How the attention kernels' roles
  * give up together (warpgroup barriers, TMEM release) is not exercised by it.
  *
- *   dev_status    int32 device word, 4-byte aligned, zeroed by the caller (a
+ *   dev_status    int32 device-visible word, 4-byte aligned, zeroed by the caller (a
  *                 nonzero word is left as it is)
  *   limit_cycles  1 .. 4,000,000,000 (the attention kernels' own limit, about
  *                 2 s at 2 GHz)

@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 // dV(u) has, and dP^T(u+1) right behind dK(u), not behind the drain's read.  14/2/64, sixteen of
 // 4,096: 3.89 ms for the serial loop with 16-byte reductions of 32 different rows that was here
 // first, 1.42 for the order of d = 128, 1.35 with dP^T ahead, 1.29 with S^T ahead too, 1.27 with the
-// drain's pace set again (247 -> 759 TFLOP/s credited).
+// drain's pace set again, 1.26 now (247 -> 767 TFLOP/s credited).
 //   WG0   warp 0: TMA producer (K and V once, NST tiles of Q and dO in flight)
 //         warp 1: TMEM allocation, MMAs of S^T and dV;  warp 2: MMAs of dP^T, dK and dQ;  warp 3: row terms
 //         (both run warp-uniformly up to an elected lane's issue, which keeps descriptors in uniform
@@ -141,6 +141,12 @@ __global__ void __launch_bounds__(256) bwd_dq_cvt(const float* __restrict__ acc,
 // TMEM (512 columns): dV, dK (D each), S^T (128), dP^T/dS^T (128).  d = 128: P^T goes over the S^T
 // columns and dQ over the dP^T columns (dK(u) reads dS^T there first, in pipe order).  d = 64: dQ
 // and P^T have 64 columns each.
+// Pipe order: the MMAs one thread issues are taken to execute in issue order.  PTX states that for MMAs
+// of one shape on one accumulator; here it is relied on where an MMA overwrites the TMEM operand of the
+// one before it, across accumulators and, at d = 64, across shapes: S^T(u+1) over the P^T that dV(u)
+// reads and dQ(u) over the dS^T that dK(u) reads (d = 128, all N = 128), dP^T(u+1) (N = 128) over the
+// dS^T that dK(u) (N = 64) reads (d = 64).  No completed barrier stands between them; the comparisons
+// with the oracle are what shows a violation.
 
 // TMEM loads / stores of N consecutive 32-bit columns of the warp's 32 lanes.
 template <int N>
@@ -197,9 +203,12 @@ struct Bwd {
   // d = 128: K^T (MN-major, M = dims) x dS (MN-major, N = queries); d = 64: dS^T x K (both MN-major)
   static constexpr uint32_t IDESC_DQ = D == 128 ? idesc_bf16(128, 128, 1, 1) : idesc_bf16(128, D, 1, 1);
 };
-static_assert(Bwd<128>::SMEM <= 232448, "shared memory budget");
-static_assert(Bwd<128>::REG_CTRL + 2 * Bwd<128>::REG_COMPUTE + Bwd<128>::REG_DRAIN <= 4 * Bwd<128>::REG_LAUNCH,
-              "setmaxnreg targets exceed the registers the block is launched with");
+static_assert(Bwd<64>::SMEM <= 232448 && Bwd<128>::SMEM <= 232448, "shared memory budget");
+template <int D>
+constexpr bool regs_fit() {
+  return Bwd<D>::REG_CTRL + 2 * Bwd<D>::REG_COMPUTE + Bwd<D>::REG_DRAIN <= 4 * Bwd<D>::REG_LAUNCH;
+}
+static_assert(regs_fit<64>() && regs_fit<128>(), "setmaxnreg targets exceed the registers the block is launched with");
 
 struct BwdBars {
   uint64_t kv_full;
@@ -991,7 +1000,7 @@ cudaError_t launch_bwd_d(const AttnArgs& a, const void* o, const float* lse, con
   char* w = static_cast<char*>(ws) + kWsHeader;
   float* dvec = reinterpret_cast<float*>(w);
   float* dq_acc = reinterpret_cast<float*>(w + align256((size_t)a.hq * a.num_tokens * 4));
-  // gathered: fp32 trajectory-layout accumulators of dQ, dK, dV after the segment-layout dQ
+  // gathered: fp32 trajectory-layout accumulators of dQ, dK, dV behind the (unused) segment-layout dQ
   float *dq_t = nullptr, *dk_t = nullptr, *dv_t = nullptr;
   const int64_t rows = a.num_tokens * a.hq;
   if (GATHER) {
@@ -1079,7 +1088,9 @@ cudaError_t launch_bwd_d(const AttnArgs& a, const void* o, const float* lse, con
 size_t attn_bwd_ws_bytes(const AttnArgs& a) {
   if (a.num_tokens < 0 || a.hq <= 0 || a.hkv <= 0 || a.d <= 0 || a.traj_tokens < 0) return kWsHeader;
   size_t b = kWsHeader + align256((size_t)a.hq * a.num_tokens * 4) + align256((size_t)a.num_tokens * a.hq * a.d * 4);
-  if (a.traj_tokens > 0)  // gathered: fp32 trajectory-layout dQ, dK, dV accumulators
+  // gathered: fp32 trajectory-layout dQ, dK, dV accumulators.  The size callers know, vcs_attn_bwd's plus
+  // these, stays: its segment-layout dQ term is unused space then.
+  if (a.traj_tokens > 0)
     b += align256((size_t)a.traj_tokens * a.hq * a.d * 4) + 2 * align256((size_t)a.traj_tokens * a.hkv * a.d * 4);
   return b;
 }

@@ -39,9 +39,10 @@
 //
 // d = 128: per K/V tile j the MMA warp issues, for each tile k once its P_k(j) is in
 // TMEM: O_k += P_k(j) V_j, then S_k(j+1) = Q_k K_{j+1}^T.  The tensor pipe
-// executes in order, so the completion of S_k(j+1) also means that P_k(j) has
-// been consumed and O_k is up to date, which is all the softmax warps wait
-// for.  The two tiles alternate, so one tile's MMAs run while the other
+// executes in order (PTX states that for MMAs of one shape on one accumulator; here
+// S_k(j+1) overwrites the P_k(j) that the MMA before it reads), so the completion of
+// S_k(j+1) also means that P_k(j) has been consumed and O_k is up to date, which is all
+// the softmax warps wait for.  The two tiles alternate, so one tile's MMAs run while the other
 // tile's softmax warps work.  The MMA thread commits only what the softmax
 // warps wait for (a commit holds it, and the pipe, about as long as an MMA);
 // the K/V ring slots are handed back to the producer by one softmax thread of
@@ -559,13 +560,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       // The K/V ring slots are handed back from here rather than by commits of the MMA thread
       // (a tcgen05.commit holds that thread, and the tensor pipe, for about as long as an MMA):
       // once S_k(j) of the last tile is complete, in-order execution has also completed every
-      // MMA that reads K_j (the S(j) of both tiles) and V_{j-1} (the P V of both tiles at
-      // step j-1), so one thread of that tile's warpgroup frees their slots.  The last V_{n-1}
+      // MMA that reads K_j (the S(j) of both tiles) and, without OWN_P, V_{j-1} (the P V of both
+      // tiles at step j-1; with OWN_P another warp issues them, and the last tile's o_done(j-1)
+      // says so), so one thread of that tile's warpgroup frees their slots.  The last V_{n-1}
       // is not handed back: the producer has issued every load by then.
       const bool releaser = (!GATHER || C::OWN_P) && (has1 ? wg == 1 : wg == 0) && quad == 0 && lane == 0;
       for (int j = 0; j <= mt; ++j) {
-        // S(j) complete also means P(j-1) was consumed and O holds P(j-1) V.  The wait's
-        // outcome is the warp's: the TMEM loads and votes below are warp-collective.
+        // Without OWN_P, S(j) complete also means P(j-1) was consumed and O holds P(j-1) V (with it, the
+        // wait for o_done below does).  The wait's outcome is the warp's: the TMEM loads and votes below
+        // are warp-collective.
         if (!mbar_wait_warp(&bars->s_full[wg], j & 1)) { ok = false; break; }
         if (releaser) {
           // ring items: K_j is 0 for j = 0, else 2j-1; V_{j-1} is 2(j-1)+2 = 2j (j-1 < nkv-1 here)
@@ -789,9 +792,11 @@ cudaError_t launch_fwd_d(const AttnArgs& a, void* o, float* lse, void* ws, cudaS
   int32_t* total = reinterpret_cast<int32_t*>(w + kWsItemTotal);
   int32_t* off = reinterpret_cast<int32_t*>(w + kWsHeader);
   int4* items = reinterpret_cast<int4*>(w + kWsHeader + align256(((size_t)a.num_segments + 1) * 4));
-  // Up to 2,048 units in 64 segments one block scans and lists them (a warp per segment, so 64 are two
-  // passes, and at most 2 units a thread): one four-step rollout through the allocating calls
-  // 455 -> 425 us, with the two header memsets that the calls' first kernels replaced.
+  // Up to 2,048 units in 64 segments one block scans and lists them, a warp per segment (64 are two
+  // passes; one segment's 1,880 units at 40/8/128, L = 12,000, are 59 a lane): one four-step rollout
+  // through the allocating calls 455 -> 425 us, with the two header memsets that the calls' first
+  // kernels replaced.  The whole forward with the list in one launch / two, us: that segment 850 / 850,
+  // two of 9,000 at 28/4/128 711 / 715, 40 of 256 at 40/8/128 106 / 113, 60 of 300 at 14/2/64 82 / 84.
   const bool one = max_items <= 2048 && a.num_segments <= 64;
   fwd_item_scan<<<1, 1024, 0, st>>>(a.cu_seqlens, a.num_segments, (int32_t)a.num_tokens, a.max_seqlen, a.hq, a.hkv,
                                     a.seg_shared, (int32_t)max_items, off, total, one ? items : nullptr, a.status);

@@ -35,7 +35,7 @@ struct SegWorkspace {
   int32_t* seg_new;     // [num_steps] global step of the first new step s_j
   int32_t* seg_last;    // [num_steps] global step of the last step e_j
   int32_t* seg_traj;    // [num_steps] trajectory of the segment
-  int64_t* totals;      // [5]: num_segments, num_tokens, max_seqlen, status, blocks done (256 bytes reserved)
+  int64_t* totals;      // [5]: num_segments, num_tokens, max_seqlen, status, blocks done
 };
 size_t seg_workspace_bytes(int32_t num_traj, int64_t num_steps);
 SegWorkspace seg_workspace_carve(void* ws, int32_t num_traj, int64_t num_steps);

@@ -401,12 +401,12 @@ size_t seg_workspace_bytes(int32_t num_traj, int64_t num_steps) {
   const size_t S = (size_t)num_steps, B = (size_t)num_traj;
   size_t n = 0;
   n += align256((S + 1) * 8) * 2;       // step_inc, txt_inc
-  n += align256(B * 4) * 2;             // traj_maxlen (and as much unused)
+  n += align256(B * 4) * 2;             // traj_maxlen; as much is reserved, so that the size stays as callers know it
   n += align256(B * 8);                 // traj_base
   n += align256((B + 1) * 8) * 2;       // seg_base, tok_base
   n += align256((S + 1) * 8);           // seg_start
   n += align256(S * 4) * 4;             // seg_full/new/last, seg_traj
-  n += align256(4 * 8);                 // totals
+  n += align256(5 * 8);                 // totals
   return n;
 }
 
@@ -419,11 +419,11 @@ SegWorkspace seg_workspace_carve(void* ws, int32_t num_traj, int64_t num_steps) 
     return r;
   };
   SegWorkspace w;
-  w.totals = reinterpret_cast<int64_t*>(take(4 * 8));
+  w.totals = reinterpret_cast<int64_t*>(take(5 * 8));
   w.step_inc = reinterpret_cast<int64_t*>(take((S + 1) * 8));
   w.txt_inc = reinterpret_cast<int64_t*>(take((S + 1) * 8));
   w.traj_maxlen = reinterpret_cast<int32_t*>(take(B * 4));
-  take(B * 4);
+  take(B * 4);  // reserved
   w.traj_base = reinterpret_cast<int64_t*>(take(B * 8));
   w.seg_base = reinterpret_cast<int64_t*>(take((B + 1) * 8));
   w.tok_base = reinterpret_cast<int64_t*>(take((B + 1) * 8));
