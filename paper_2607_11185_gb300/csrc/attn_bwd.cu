@@ -174,7 +174,7 @@ struct Bwd {
   static constexpr int OFF_QD = 2 * TILE;
   static constexpr int OFF_DS = OFF_QD + 2 * NST * TILE;  // dS^T [128 keys][128 queries], two 64-query blocks
   static constexpr int NDS = D == 128 ? 1 : 2;              // buffers of dS^T, by tile parity
-  static constexpr int OFF_ROW = OFF_DS + NDS * 2 * BLOCK;  // [tile parity][WG k]: -lse*log2e of 64 queries, -D*scale
+  static constexpr int OFF_ROW = OFF_DS + NDS * 2 * BLOCK;  // [tile parity][WG k]: -lse*log2e of 64 queries, -D (* scale)
   static constexpr int OFF_BAR = OFF_ROW + 2 * 2 * 128 * 4;
   static constexpr int BAR_BYTES = 512;
   static constexpr int SMEM = OFF_BAR + BAR_BYTES;
@@ -191,6 +191,7 @@ struct Bwd {
   // Row terms staged by warp 3, or by the compute warps.  d = 64, which the compute warps bound: 1.34
   // ms against 1.29 (14/2/64, sixteen segments of 4,096); d = 128: 0.5% slower by a warp of its own.
   static constexpr bool ROW_WARP = D == 64;
+  static constexpr bool SCALED_D = D == 128;
   static constexpr int REG_CTRL = ROW_WARP ? 96 : 80, REG_COMPUTE = ROW_WARP ? 136 : 144, REG_DRAIN = 144;
   static constexpr int REG_LAUNCH = 65536 / THREADS;
   // Tile u's Q and dO take the slots 2(u % NST) and the next, in turn: dO(u) is released well
@@ -371,6 +372,10 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       dd = __ldg(&dvec[j]);
     }
   };
+
+  // -D, scaled at d = 128, where dS = P fma(dP, scale, -D scale).  d = 64 keeps the exact difference,
+  // dS = P (dP - D) scale: a rounded D scale would leave a residue where dP and D cancel.
+  auto nd_of = [&](float dd) { return C::SCALED_D ? -dd * scale : -dd; };
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sbase = smem_u32(smem);
@@ -597,7 +602,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       if (!ok) abort_now();
     } else if (C::ROW_WARP && warp == 3) {
       // ---------------------------------------------------------- row terms
-      // Stages -lse*log2e and -D*scale of each tile's 128 queries for the compute warps, loaded a tile
+      // Stages -lse*log2e and -D of each tile's 128 queries for the compute warps, loaded a tile
       // ahead (behind the drain's reductions a load can take more than a tile's time), and joins S^T's
       // barrier, so that the compute warps wait once for both.
       Walk w = walk0;
@@ -616,7 +621,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         for (int i = 0; i < 4; ++i) {  // half i/2 of warpgroup i%2's 64 queries: nl, then nd
           float* r = rows + (u & 1) * 256 + (i & 1) * 128 + (i >> 1) * 32 + lane;
           r[0] = -l[i] * 1.4426950408889634f;
-          r[64] = -dd[i] * scale;
+          r[64] = nd_of(dd[i]);
         }
         load();
         __syncwarp();
@@ -635,7 +640,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
     const int quad = warp & 3;
     const int r = quad * 32 + lane;  // TMEM lane: key row
     const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-    // row terms of the warpgroup's 64 queries: nl = -lse*log2e, then nd = -D*scale; two buffers
+    // row terms of the warpgroup's 64 queries: nl = -lse*log2e, then nd (nd_of D); two buffers
     const uint32_t rt_u32 = smem_u32(smem + C::OFF_ROW) + k * 512;
     const uint32_t ds_row = sbase + C::OFF_DS + r * 128;
     const uint64_t sl2 = f2pack(scale_log2, scale_log2), sc2 = f2pack(scale, scale);
@@ -663,7 +668,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
       if constexpr (!C::ROW_WARP) {
         if (tw < 64) {
           rt_s[(u & 1) * 256 + tw] = -l0 * 1.4426950408889634f;
-          rt_s[(u & 1) * 256 + 64 + tw] = -d0 * scale;
+          rt_s[(u & 1) * 256 + 64 + tw] = nd_of(d0);
         }
         l0 = l1;
         d0 = d1;
@@ -739,7 +744,7 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
         continue;
       }
       tc_fence_after();
-      // dS^T = P^T (dP^T - D) * scale, 16 columns at a time, the next ones' loads in flight
+      // dS^T = P^T (dP^T - D) scale, 16 columns at a time, the next ones' loads in flight
       uint32_t dp[2][16];
       tmem_ld_cols<16>(trow + C::TM_P + 32 * k, dp[0]);
       tmem_ld_wait();
@@ -756,12 +761,12 @@ __global__ void __launch_bounds__(Bwd<D>::THREADS, 1)
 #pragma unroll
         for (int c = 0; c < 16; c += 2) {
           const uint4 t = rq[cur][c / 4];
-          const uint64_t y =
-              ffma2(f2pack(__uint_as_float(dp[cur][c]), __uint_as_float(dp[cur][c + 1])), sc2,
-                    f2pack(__uint_as_float(c & 2 ? t.z : t.x), __uint_as_float(c & 2 ? t.w : t.y)));
+          const uint64_t x = f2pack(__uint_as_float(dp[cur][c]), __uint_as_float(dp[cur][c + 1]));
+          const uint64_t nd = f2pack(__uint_as_float(c & 2 ? t.z : t.x), __uint_as_float(c & 2 ? t.w : t.y));
           const int pc = 16 * (ch & 1) + c;
+          const uint64_t pp = f2pack(__uint_as_float(p[ch >> 1][pc]), __uint_as_float(p[ch >> 1][pc + 1]));
           float a, b;
-          f2unpack(fmul2(f2pack(__uint_as_float(p[ch >> 1][pc]), __uint_as_float(p[ch >> 1][pc + 1])), y), a, b);
+          f2unpack(C::SCALED_D ? fmul2(pp, ffma2(x, sc2, nd)) : fmul2(fmul2(pp, fadd2(x, nd)), sc2), a, b);
           wd[c / 2] = pack_bf16(a, b);
         }
 #pragma unroll

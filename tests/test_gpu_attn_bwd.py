@@ -277,3 +277,21 @@ def test_segment_ends_around_the_drains_row_groups(d):
     got = vcs.attn_bwd_gathered(q, k, v, gat, o, lse, do, torch.from_numpy(cu).cuda(), max(lengths))
     for name, a, b in zip(("dq", "dk", "dv"), got, grads):
         assert (a.double() - b.double()).norm() <= 5e-3 * b.double().norm(), name
+
+
+def test_d64_keeps_the_exact_difference_of_dp_and_d():
+    """One-token segments: P = 1, O = v and dP = D exactly for small whole numbers, so dS, and with it dQ
+    and dK, is 0, at any scale.  (-D scale) rounded on its own left a residue at scales that are not a
+    power of two."""
+    from paper_2607_11185_gb300 import vcs
+    n, d = 9, 64
+    g = torch.Generator(device="cuda").manual_seed(4)
+    q, k = (torch.randn((n, h, d), generator=g, device="cuda").bfloat16() for h in (2, 1))
+    v, do = (torch.randint(-3, 4, (n, h, d), generator=g, device="cuda").bfloat16() for h in (1, 2))
+    cu = torch.arange(n + 1, dtype=torch.int32, device="cuda")
+    for scale in (0.1, 0.3, 0.125):
+        o, lse = vcs.attn_fwd(q, k, v, cu, 1, softmax_scale=scale)
+        assert torch.equal(o, v.expand(n, 2, d))
+        dq, dk, dv = vcs.attn_bwd(q, k, v, o, lse, do, cu, 1, softmax_scale=scale)
+        assert not dq.any() and not dk.any()
+        assert torch.equal(dv.float(), do.float().sum(1, keepdim=True))
