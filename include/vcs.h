@@ -97,7 +97,9 @@ size_t vcs_segments_workspace_size(int32_t num_traj, int64_t num_steps);
  *   sizes     device-visible output: segment count, segment-token count,
  *             longest segment, device status (VCS_ERR_DEVICE_CHECK for
  *             inconsistent cu_steps or negative counts, VCS_ERR_OVERFLOW when
- *             a token count exceeds INT32_MAX)
+ *             a token count exceeds INT32_MAX; of overlapping trajectories,
+ *             which only inconsistent cu_steps describe, the other three
+ *             values mean nothing and may differ from call to call)
  *   ws        device workspace of vcs_segments_workspace_size() bytes
  * Asynchronous: synchronise `stream` before reading *sizes. */
 vcs_status vcs_plan_segments(const int32_t* cu_steps, int32_t num_traj, int64_t num_steps,
