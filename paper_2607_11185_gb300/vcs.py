@@ -12,8 +12,6 @@ non-zero status.
 from __future__ import annotations
 
 import ctypes
-import functools
-import inspect
 import math
 import os
 from typing import Optional
@@ -301,34 +299,24 @@ def _tensors(x):
             yield from _tensors(y)
 
 
-def _on_stream(fn):
-    """Runs a convenience with its `stream` as the current one, so that the workspace and the outputs come
-    from that stream's memory pool and the status words are read in that stream's order.  The outputs are
+def _on_stream(given, fn, *args, **kwargs):
+    """fn(...) with the stream `given` as the current one, so that the workspace and the outputs come from
+    that stream's memory pool and the status words are read in that stream's order.  The outputs are
     marked as used by the caller's current stream, where the caller goes on with them."""
-    at = list(inspect.signature(fn).parameters).index("stream")
-
-    @functools.wraps(fn)
-    def call(*args, **kwargs):
-        given = args[at] if len(args) > at else kwargs.pop("stream", None)
-        if given is None:
-            return fn(*args, **kwargs)
-        if len(args) > at:
-            args = (*args[:at], None, *args[at + 1:])
-        caller, stream = torch.cuda.current_stream(), _torch_stream(given)
-        if stream == caller:
-            return fn(*args, **kwargs)
-        with torch.cuda.stream(stream):
-            out = fn(*args, **kwargs)
-        for t in _tensors(out):
-            t.record_stream(caller)
-        return out
-
-    return call
+    caller, stream = torch.cuda.current_stream(), _torch_stream(given)
+    if stream == caller:
+        return fn(*args, **kwargs)
+    with torch.cuda.stream(stream):
+        out = fn(*args, **kwargs)
+    for t in _tensors(out):
+        t.record_stream(caller)
+    return out
 
 
-@_on_stream
 def plan_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, stream=None):
     """Segment count, token count and longest segment (synchronises once)."""
+    if stream is not None:
+        return _on_stream(stream, plan_segments, cu_steps, step_img, step_txt, window, keep)
     dev = cu_steps.device
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
     nb = vcs_segments_workspace_size(num_traj, num_steps)
@@ -344,10 +332,11 @@ def _plan(cu_steps, num_traj, num_steps, step_img, step_txt, window, keep, ws, n
     return ns, nt, tail & 0xFFFFFFFF
 
 
-@_on_stream
 def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, with_mask: bool = True,
                    stream=None):
     """Plan + build: returns a dict of device tensors and the sizes."""
+    if stream is not None:
+        return _on_stream(stream, build_segments, cu_steps, step_img, step_txt, window, keep, with_mask)
     dev = cu_steps.device
     num_traj, num_steps = cu_steps.numel() - 1, step_img.numel()
     nb = vcs_segments_workspace_size(num_traj, num_steps)
@@ -368,8 +357,9 @@ def build_segments(cu_steps, step_img, step_txt, window: int, keep: int = 0, wit
     return out
 
 
-@_on_stream
 def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
+    if stream is not None:
+        return _on_stream(stream, gather, q_traj, k_traj, v_traj, tok_gather)
     nt = tok_gather.numel()
     _, hq, d = q_traj.shape
     hkv = k_traj.shape[1]
@@ -384,8 +374,9 @@ def gather(q_traj, k_traj, v_traj, tok_gather, stream=None):
     return q, k, v
 
 
-@_on_stream
 def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, stream=None, check=True):
+    if stream is not None:
+        return _on_stream(stream, attn_fwd, q, k, v, cu_seqlens, max_seqlen, softmax_scale, check=check)
     nt, hq, d = q.shape
     hkv = k.shape[1]
     ns = cu_seqlens.numel() - 1
@@ -400,9 +391,10 @@ def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, s
     return o, lse
 
 
-@_on_stream
 def attn_bwd(q, k, v, o, lse, dout, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0, stream=None,
              check=True):
+    if stream is not None:
+        return _on_stream(stream, attn_bwd, q, k, v, o, lse, dout, cu_seqlens, max_seqlen, softmax_scale, check=check)
     nt, hq, d = q.shape
     hkv = k.shape[1]
     ns = cu_seqlens.numel() - 1
@@ -416,9 +408,10 @@ def attn_bwd(q, k, v, o, lse, dout, cu_seqlens, max_seqlen: int, softmax_scale: 
     return dq, dk, dv
 
 
-@_on_stream
 def shared_prefix(cu_seqlens, seg_traj, tok_gather, stream=None):
     """Per segment, its common prefix length with the previous segment of its trajectory."""
+    if stream is not None:
+        return _on_stream(stream, shared_prefix, cu_seqlens, seg_traj, tok_gather)
     ns = cu_seqlens.numel() - 1
     out = torch.empty(max(ns, 0), dtype=torch.int32, device=cu_seqlens.device)
     status = _host_words(1, torch.int32)
@@ -428,10 +421,12 @@ def shared_prefix(cu_seqlens, seg_traj, tok_gather, stream=None):
     return out
 
 
-@_on_stream
 def attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, max_seqlen: int, softmax_scale: float = 0.0, stream=None,
                    check=True):
     """vcs_attn_fwd's o and lse, computing each shared prefix row once per trajectory."""
+    if stream is not None:
+        return _on_stream(stream, attn_fwd_reuse, q, k, v, cu_seqlens, seg_shared, max_seqlen, softmax_scale,
+                          check=check)
     nt, hq, d = q.shape
     hkv = k.shape[1]
     ns = cu_seqlens.numel() - 1
@@ -446,11 +441,13 @@ def attn_fwd_reuse(q, k, v, cu_seqlens, seg_shared, max_seqlen: int, softmax_sca
     return o, lse
 
 
-@_on_stream
 def attn_fwd_gathered(q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen: int, softmax_scale: float = 0.0,
                       stream=None, check=True):
     """Attention forward over the segments, reading trajectory-layout q/k/v through tok_gather;
     o [num_tokens, hq, d] and lse [hq, num_tokens] in segment layout."""
+    if stream is not None:
+        return _on_stream(stream, attn_fwd_gathered, q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen,
+                          softmax_scale, check=check)
     tt, hq, d = q_traj.shape
     hkv = k_traj.shape[1]
     nt = tok_gather.numel()
@@ -466,11 +463,13 @@ def attn_fwd_gathered(q_traj, k_traj, v_traj, tok_gather, cu_seqlens, max_seqlen
     return o, lse
 
 
-@_on_stream
 def attn_bwd_gathered(q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqlens, max_seqlen: int,
                       softmax_scale: float = 0.0, stream=None, check=True):
     """Attention backward over the segments with trajectory-layout q/k/v read through tok_gather;
     returns dq, dk, dv in trajectory layout (each token's segment copies summed)."""
+    if stream is not None:
+        return _on_stream(stream, attn_bwd_gathered, q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqlens,
+                          max_seqlen, softmax_scale, check=check)
     tt, hq, d = q_traj.shape
     hkv = k_traj.shape[1]
     nt = tok_gather.numel()
@@ -486,11 +485,13 @@ def attn_bwd_gathered(q_traj, k_traj, v_traj, tok_gather, o, lse, dout, cu_seqle
     return dq, dk, dv
 
 
-@_on_stream
 def grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv, eps_low: float = 0.2,
               eps_high: float = 0.28, clip_cap: float = 3.0, kl_coef: float = 1e-4, with_grad: bool = True,
               stream=None, check=True):
     """Loss (fp64 device scalar) and d loss / d logp (fp32, or None)."""
+    if stream is not None:
+        return _on_stream(stream, grpo_loss, logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv,
+                          eps_low, eps_high, clip_cap, kl_coef, with_grad, check=check)
     nt = logp.numel()
     dev = logp.device
     loss = torch.empty(1, dtype=torch.float64, device=dev)
@@ -505,9 +506,10 @@ def grpo_loss(logp, old_logp, ref_logp, tok_loss_mask, cu_seqlens, seg_traj, adv
     return loss, dlogp
 
 
-@_on_stream
 def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     """(ids int32, logp fp32) of every segment token (Algorithm 1's stream fields)."""
+    if stream is not None:
+        return _on_stream(stream, stream_fields, traj_ids, traj_logp, tok_gather, tok_loss_mask)
     nt = tok_gather.numel()
     dev = tok_gather.device
     ids = torch.empty(nt, dtype=torch.int32, device=dev)
@@ -519,9 +521,10 @@ def stream_fields(traj_ids, traj_logp, tok_gather, tok_loss_mask, stream=None):
     return ids, logp
 
 
-@_on_stream
 def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     """Indices of the trainable tokens in order (int32 device tensor)."""
+    if stream is not None:
+        return _on_stream(stream, compact_trainable, tok_loss_mask, capacity)
     nt = tok_loss_mask.numel()
     dev = tok_loss_mask.device
     cap = nt if capacity is None else capacity
@@ -534,8 +537,9 @@ def compact_trainable(tok_loss_mask, capacity=None, stream=None):
     return idx[: count.tolist()[0]]
 
 
-@_on_stream
 def group_advantage(rewards, group_size: int, eps: float = 1e-6, stream=None):
+    if stream is not None:
+        return _on_stream(stream, group_advantage, rewards, group_size, eps)
     adv = torch.empty_like(rewards)
     _check(vcs_group_advantage(rewards, rewards.numel() // group_size, group_size, eps, adv),
            "vcs_group_advantage")
