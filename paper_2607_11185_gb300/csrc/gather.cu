@@ -134,16 +134,21 @@ cudaError_t launch_gather(const void* q_src, const void* k_src, const void* v_sr
   const int64_t cap = 152 * 16;
   const int64_t q_chunks = q_row_bytes / 16, kv_chunks = kv_row_bytes / 16;
   if (q_chunks < kNarrow && kv_chunks < kNarrow) {
-    // as many tokens a warp as leave 32 warps an SM a share, but no fewer than fill a step
-    int64_t per_warp = (num_tokens + 152 * 32 - 1) / (152 * 32);
+    // At most 32 tokens a warp, and as many as divide the tokens evenly over whole passes of the 32 warps an
+    // SM holds (174,000 tokens at 4/4/64: 102 us, 127 with 32 a warp, which leave a second pass nearly
+    // empty; 111 for a chunk a thread), in fours where they are many, whose chunks fill whole steps more
+    // often, but no fewer than fill a step.
+    const int64_t slots = 152 * 32, passes = (num_tokens + slots * 32 - 1) / (slots * 32);
+    int64_t per_warp = (num_tokens + slots * passes - 1) / (slots * passes);
+    if (per_warp > 16) per_warp = (per_warp + 3) / 4 * 4;
     if (per_warp * q_chunks < 32) per_warp = (31 + q_chunks) / q_chunks;
     if (per_warp > 32) per_warp = 32;
-    const int64_t warps = (num_tokens + per_warp - 1) / per_warp;
-    int64_t blocks = (warps + kThreads / 32 - 1) / (kThreads / 32);
-    if (blocks > cap) blocks = cap;
+    const bool few_steps = q_chunks + 2 * kv_chunks < kUnroll;
+    int64_t blocks = ((num_tokens + per_warp - 1) / per_warp + kThreads / 32 - 1) / (kThreads / 32);
+    if (few_steps && blocks > cap) blocks = cap;
     auto magic = [](int64_t c) { return c > 0 ? (1u << kMagicShift) / (uint32_t)c + 1 : 0u; };
     // of a few steps a pass none waits for another, and more warps fit (Q alone, a chunk a row: 20.5 -> 16.4 us)
-    const auto kernel = q_chunks + 2 * kv_chunks < kUnroll ? gather_narrow<1> : gather_narrow<kUnroll>;
+    const auto kernel = few_steps ? gather_narrow<1> : gather_narrow<kUnroll>;
     kernel<<<(unsigned)blocks, kThreads, 0, st>>>(
         static_cast<const int4*>(q_src), static_cast<const int4*>(k_src), static_cast<const int4*>(v_src), traj_tokens,
         tok_gather, num_tokens, (int)q_chunks, (int)kv_chunks, magic(q_chunks), magic(kv_chunks), (int)per_warp,
